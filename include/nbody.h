@@ -406,9 +406,18 @@ enum {
 int nbody_tile_info(int32_t law, int32_t tile, int32_t *threads, int32_t *i_per_thread,
                     int32_t *j_lanes, int32_t *j_tile, int32_t *kind);
 /* Install the tuned (tile, jsplit) for (tile table law, n-bucket); bucket =
- * floor(log2 n) (the batched table uses bucket 0). Used by params->tile == -1. */
+ * floor(log2 n) (the batched table uses bucket 0). Used by params->tile == -1;
+ * tile -1 removes the entry. */
 int nbody_set_tuned(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit);
-/* Query the configuration a call with (law, n) and tile == -1 would use. */
+/* The same for an entry of a stored table, which does not stand in the way of the
+ * streamed kernels: calls with tile == -1 and jsplit == 0 for which the library has
+ * one (nbody_forces and nbody_step without NBODY_FIXED_POINT) run that unless
+ * nbody_set_tuned or nbody_tune installed an entry for the size; the other calls
+ * (subsets, nbody_forces_static, a j-split of the caller's, sizes whose partial sums
+ * would pass the limit) take the stored tile. */
+int nbody_set_stored(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit);
+/* Query the tile-table entry of (law, n): the installed or stored one, else the
+ * table's default row. */
 int nbody_get_config(int32_t law, int64_t n, int32_t *tile, int32_t *jsplit);
 /* Device scratch bytes a call of nbody_forces / nbody_step with these params
  * and n requests from the library's per-(device, stream) workspace: the
@@ -427,7 +436,8 @@ int nbody_workspace_size(const nbody_params *params, int64_t n, int32_t report_r
  * 32} that fits n (Newton-symmetric tiles: the splits their plan takes, and only
  * where their partial-sum cap admits n) is run once to warm up and `reps` (1..1000) more times, timed
  * with CUDA events on `stream`; the median decides. The fastest is installed
- * with nbody_set_tuned for bucket floor(log2 n) and returned in best_tile,
+ * with nbody_set_tuned for bucket floor(log2 n) (with nbody_set_stored where the
+ * library's streamed kernel is faster still) and returned in best_tile,
  * best_jsplit and best_ms (milliseconds per call; any may be NULL). What is
  * timed: tables 0-2 nbody_forces (law = table), 4 nbody_forces with
  * NBODY_FIXED_POINT (eps2 > 0), 5 / 6 / 8 nbody_adjoint (gravity / LJC / LJC

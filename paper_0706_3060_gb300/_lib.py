@@ -43,7 +43,8 @@ EXPORTS = (
     "nbody_pack_grav", "nbody_pack_ljc", "nbody_forces", "nbody_step",
     "nbody_batch_plan_create", "nbody_batch_plan_destroy", "nbody_batch_plan_particles",
     "nbody_batch_run", "nbody_forces_batched", "nbody_adjoint", "nbody_adjoint_leapfrog",
-    "nbody_tile_count", "nbody_tile_info", "nbody_set_tuned", "nbody_get_config",
+    "nbody_tile_count", "nbody_tile_info", "nbody_set_tuned", "nbody_set_stored",
+    "nbody_get_config",
     "nbody_timing_enable", "nbody_timing_read", "nbody_peak_probe", "nbody_forces_static",
     "nbody_forces_subset", "nbody_forces_jerk", "nbody_hermite_step", "nbody_selftest_timeout",
     "nbody_tune", "nbody_workspace_size",
@@ -118,6 +119,7 @@ def load(path: str | None = None):
                                  ctypes.POINTER(i32), ctypes.POINTER(i32), ctypes.POINTER(i32)],
                                 ctypes.c_int),
             "nbody_set_tuned": ([i32, i32, i32, i32], ctypes.c_int),
+            "nbody_set_stored": ([i32, i32, i32, i32], ctypes.c_int),
             "nbody_timing_enable": ([i32], ctypes.c_int),
             "nbody_peak_probe": ([i32, i32, ctypes.POINTER(f64), ctypes.POINTER(f64)],
                                  ctypes.c_int),

@@ -15,7 +15,10 @@ namespace nbody {
 
 int launch_finalize(const FinalizeArgs &f, cudaStream_t s, int *nblk_out, bool pdl) {
   const int nblk = std::max(1, (f.n + kFinThreads - 1) / kFinThreads);
-  NB_CUDA(launch_kernel(finalize_kernel, nblk, kFinThreads, 0, s, pdl, f));
+  if (f.tri.h > 0)
+    NB_CUDA(launch_kernel(finalize_kernel<kFinSplit>, nblk, kFinThreads * kFinSplit, 0, s, pdl, f));
+  else
+    NB_CUDA(launch_kernel(finalize_kernel<1>, nblk, kFinThreads, 0, s, pdl, f));
   if (nblk_out) *nblk_out = nblk;
   return NBODY_OK;
 }
@@ -108,7 +111,8 @@ struct ScratchSizes {
 
 ScratchSizes scratch_sizes(int law, int n, const Plan1 &plan, int diag_rows) {
   ScratchSizes z{};
-  const bool lo = !plan.atomic && (!plan.tile->sym || plan.tile->fixed);  // FX: int64 (z, w)
+  // FX: int64 (z, w)
+  const bool lo = !plan.atomic && !plan.tri && (!plan.tile->sym || plan.tile->fixed);
   const int64_t jn = plan.tile->sym ? int64_t(plan.slices) * plan.slice_len : n;
   z.part = plan.atomic ? round_up(size_t(8) * size_t(n) * sizeof(long long), 256)
                        : round_up(size_t(plan.slices) * size_t(n) * sizeof(float4), 256);
@@ -116,7 +120,7 @@ ScratchSizes scratch_sizes(int law, int n, const Plan1 &plan, int diag_rows) {
   const int nblk = std::max(1, (n + kFinThreads - 1) / kFinThreads);
   z.dpart = round_up(size_t(nblk) * kDiagFields * sizeof(double), 256);
   z.drows = round_up(size_t(std::max(diag_rows, 1)) * kDiagFields * sizeof(double), 256);
-  z.jb = jbuf_bytes(law, jn);
+  z.jb = plan.tri ? 0 : jbuf_bytes(law, jn);
   z.msum = plan.atomic ? round_up(size_t((n + 511) / 512) * sizeof(double), 256) : 0;
   return z;
 }
@@ -185,6 +189,7 @@ int eval_and_finalize(const float4 *pos, const float4 *prm, const nbody_params &
   f.plain = (p.flags & NBODY_NO_COMPENSATION) ? 1 : 0;
   const bool prep = prepare_next && plan.tile->packed && (f.mode & kFinKickDrift);
   f.jnext = prep ? sc.jbuf : nullptr;
+  f.tri = plan.tri ? plan.geom : TriGeom{};
   f.jn_block = plan.tile->sym ? plan.tile->tile_i : 0;
   f.jn_words = p.law == NBODY_LAW_GRAV ? 2 : 3;
   f.rezero = (prep && plan.atomic) ? 1 : 0;
@@ -505,7 +510,12 @@ int nbody_tile_info(int32_t law, int32_t tile, int32_t *threads, int32_t *i_per_
 
 int nbody_set_tuned(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit) {
   clear_error();
-  return set_tuned(law, log2n, tile, jsplit);
+  return set_tuned(law, log2n, tile, jsplit, true);
+}
+
+int nbody_set_stored(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit) {
+  clear_error();
+  return set_tuned(law, log2n, tile, jsplit, false);
 }
 
 int nbody_get_config(int32_t law, int64_t n, int32_t *tile, int32_t *jsplit) {

@@ -36,6 +36,7 @@ std::map<int, int> g_checked;  // device -> sms
 struct Tuned {
   int tile = -1;
   int jsplit = 0;
+  bool by_caller = false;  // installed through the C ABI, not from the stored table
 };
 Tuned g_tuned[kTables][64];
 
@@ -275,7 +276,7 @@ const TileDesc *tiles_for(int law, int *count) {
   return mixed_tiles(count);
 }
 
-int set_tuned(int law, int log2n, int tile, int jsplit) {
+int set_tuned(int law, int log2n, int tile, int jsplit, bool by_caller) {
   if (law < 0 || law >= kTables || log2n < 0 || log2n >= 64)
     return set_error_msg(NBODY_EINVAL, "bad law %d or log2n %d", law, log2n);
   int count = 0;
@@ -285,6 +286,7 @@ int set_tuned(int law, int log2n, int tile, int jsplit) {
   std::lock_guard<std::mutex> lk(g_mu);
   g_tuned[law][log2n].tile = tile;
   g_tuned[law][log2n].jsplit = jsplit;
+  g_tuned[law][log2n].by_caller = by_caller && tile >= 0;
   return NBODY_OK;
 }
 
@@ -292,6 +294,19 @@ static int log2_floor(int64_t n) {
   int b = 0;
   while ((int64_t(1) << (b + 1)) <= n && b < 62) ++b;
   return b;
+}
+
+bool tuned_by_caller(int law, int64_t n) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  return g_tuned[law][log2_floor(n > 0 ? n : 1)].by_caller;
+}
+
+void tuned_entry(int law, int log2n, int *tile, int *jsplit, bool *by_caller) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  const Tuned &t = g_tuned[law][log2n];
+  *tile = t.tile;
+  *jsplit = t.jsplit;
+  *by_caller = t.by_caller;
 }
 
 // Default tile when nothing is tuned: big register blocks for large N, j-lanes
@@ -357,14 +372,51 @@ bool sym_fits(int64_t n, int block) {
 
 bool sym_atomic_law(int law) { return law == NBODY_LAW_GRAV || law == kTableGravFixed; }
 
+bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out) {
+  // Below about 2500 particles a row or two of targets cannot fill the GPU and the
+  // finalize is a launch more than the one-sided tiles' work is worth (steps at 2048:
+  // gravity 11.2 us against 9.0, LJC 11.0 both; at 4001: 15.7 against 21.7, 18.1
+  // against 30.5).
+  if (law < 0 || law > NBODY_LAW_LJC_LINEAR || n < 2500 || n > 0x7fffffffLL - 64 * 64 ||
+      tuned_by_caller(law, n))
+    return false;
+  const TriDesc *d = law == NBODY_LAW_GRAV ? tri_grav(n)
+                     : law == NBODY_LAW_LJC ? tri_ljc(n)
+                                            : tri_ljclin(n);
+  const TriGeom g = tri_geom(int(n), d->h, sms * d->per_sm);
+  const int slots = g.nb + tri_max_row_shares(g);
+  const double bytes = double(slots) * double(n) * sizeof(float4);
+  // Softened gravity from 65536 particles stays with the block-pair tiles, whose
+  // partials are added exactly in fixed point with integer atomics (64 bytes a
+  // particle): as fast there (steps at 65536: 1162 us against 1167, at 262144 17.72 ms
+  // against 17.8), where the slots would grow as n^2 (134 MB and 2.1 GB).
+  if (law == NBODY_LAW_GRAV && atomic_ok && n >= 65536) return false;
+  if (bytes > sym_part_cap()) return false;
+  // The plan's tile: none of a table, reads the positions directly.
+  static const TileDesc direct{};
+  out->tile = &direct;
+  out->tri = d;
+  out->geom = g;
+  out->slices = slots;
+  out->slice_len = 0;
+  out->n_itiles = g.nb;
+  out->grid = g.nshare;
+  out->sym_split = 1;
+  out->atomic = false;
+  return true;
+}
+
 int plan_single(int law, int64_t n, int tile, int jsplit, int sms, Plan1 *out, bool allow_sym,
                 bool atomic_ok) {
+  if (tile < 0 && jsplit <= 0 && allow_sym && plan_tri(law, n, sms, atomic_ok, out))
+    return NBODY_OK;
   return plan_targets(law, n, n, tile, jsplit, sms, out, allow_sym, atomic_ok);
 }
 
 int plan_targets(int law, int64_t n_t, int64_t n, int tile, int jsplit, int sms, Plan1 *out,
                  bool allow_sym, bool atomic_ok) {
   out->atomic = false;
+  out->tri = nullptr;
   if (law < 0 || law >= kTableVjpGrav)
     return set_error_msg(NBODY_EINVAL, "tile table %d is not a force table", law);
   int count = 0;
@@ -588,6 +640,25 @@ int launch_forces(const float4 *pos, const float4 *prm, int law, uint32_t flags,
                                         !at->ticket || !at->scale || !at->inv)))
     return set_error_msg(NBODY_EINVAL, "atomic plan and accumulators must come together");
   if (atomic) fscale = at->scale;
+  if (p.tri) {  // streamed triangle kernel: reads pos / prm themselves
+    if (tg || kd || atomic)
+      return set_error_msg(NBODY_EINVAL, "the streamed kernels take all targets as they are");
+    TriArgs t{};
+    t.p0 = pos;
+    t.p1 = prm;
+    t.part = part_hi;
+    t.eps2 = eps2;
+    t.geom = p.geom;
+    t.pdl = chained ? 1 : 0;
+    const TimerMark tm = timed ? timer_begin(0, s) : TimerMark{};
+    const cudaError_t e = p.tri->launch(t, pot, (flags & NBODY_PRECISE_RSQRT) != 0, s);
+    timer_end(tm, s);
+    if (e != cudaSuccess)
+      return set_error_msg(e == cudaErrorNoKernelImageForDevice ? NBODY_EUNSUPPORTED
+                                                                : NBODY_ECUDA,
+                           "force kernel launch failed: %s", cudaGetErrorString(e));
+    return NBODY_OK;
+  }
   if ((p.tile->fixed || p.atomic) != (fscale != nullptr))
     return set_error_msg(NBODY_EINVAL, "fixed-point tile and scale must come together");
   if (sources_ready && (!p.tile->packed || tg || (atomic && at->form_scale)))

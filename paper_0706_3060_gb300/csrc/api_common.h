@@ -15,6 +15,7 @@
 
 #include "nbody.h"
 #include "tiles.h"
+#include "tri_tiles.h"
 
 namespace nbody {
 
@@ -90,6 +91,8 @@ struct Plan1 {
   int n_itiles;
   int grid;
   int sym_split;   // symmetric tiles: source parts per block (1 otherwise)
+  const TriDesc *tri;  // streamed triangle kernel (tri_kernel.cuh) instead of the tile,
+  TriGeom geom;        // its shares (`slices` is then its slot count), or null
   bool atomic;     // symmetric gravity: per-block partials added with integer atomics
                    // into fixed-point accumulators per particle (scratch 64 bytes
                    // per particle) instead of one slot per block
@@ -111,6 +114,10 @@ int plan_single(int law, int64_t n, int tile, int jsplit, int sms, Plan1 *out,
 // Same for n_t targets against n sources (i-tiles over targets, j-slices over sources).
 int plan_targets(int law, int64_t n_t, int64_t n, int tile, int jsplit, int sms, Plan1 *out,
                  bool allow_sym = false, bool atomic_ok = false);
+// The streamed triangle kernel for a call that leaves the configuration to the
+// library, or false where a tile runs: an entry of the tile table that the caller
+// installed (nbody_set_tuned, nbody_tune), or a partial-sum buffer above its limit.
+bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out);
 // Whether the symmetric tiles of tile table `law` can accumulate atomically
 // (gravity and fixed-point gravity).
 bool sym_atomic_law(int law);
@@ -176,7 +183,11 @@ int launch_forces(const float4 *pos, const float4 *prm, int law, uint32_t flags,
 
 size_t round_up(size_t x, size_t a);
 
-int set_tuned(int law, int log2n, int tile, int jsplit);
+// by_caller: installed through the C ABI's nbody_set_tuned or nbody_tune, and then
+// preferred to the streamed kernels; otherwise a stored entry.
+int set_tuned(int law, int log2n, int tile, int jsplit, bool by_caller);
+bool tuned_by_caller(int law, int64_t n);
+void tuned_entry(int law, int log2n, int *tile, int *jsplit, bool *by_caller);
 int get_config(int law, int64_t n, int *tile, int *jsplit);
 const char *last_error_text();
 void release_all();

@@ -52,6 +52,35 @@ int run_once(int table, const void *pos, const void *prm, int64_t n, float eps2,
   }
 }
 
+// Median time of `reps` runs of call(), each between two events on `s`.
+template <class F>
+int time_call(int reps, std::vector<float> &ts, float *median, cudaStream_t s, F &&call) {
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  NB_CUDA(cudaEventCreate(&e0));
+  if (cudaEventCreate(&e1) != cudaSuccess) {
+    cudaEventDestroy(e0);
+    return set_error_msg(NBODY_ECUDA, "cudaEventCreate failed");
+  }
+  int st = NBODY_OK;
+  bool ev_fail = false;
+  for (int r = 0; r < reps && st == NBODY_OK && !ev_fail; ++r) {
+    ev_fail = cudaEventRecord(e0, s) != cudaSuccess;
+    if (!ev_fail) st = call();
+    if (!ev_fail && st == NBODY_OK)
+      ev_fail = cudaEventRecord(e1, s) != cudaSuccess ||
+                cudaEventSynchronize(e1) != cudaSuccess ||
+                cudaEventElapsedTime(&ts[size_t(r)], e0, e1) != cudaSuccess;
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (ev_fail) return set_error_msg(NBODY_ECUDA, "timing events failed");
+  if (st != NBODY_OK) return st;
+  std::vector<float> sorted(ts);
+  std::nth_element(sorted.begin(), sorted.begin() + reps / 2, sorted.end());
+  *median = sorted[size_t(reps / 2)];
+  return NBODY_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -90,14 +119,7 @@ int nbody_tune(int32_t table, const void *pos_m, const void *prm, int64_t n, flo
 
   int count = 0;
   const TileDesc *tiles = tiles_for(table, &count);
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  NB_CUDA(cudaEventCreate(&e0));
-  if (cudaEventCreate(&e1) != cudaSuccess) {
-    cudaEventDestroy(e0);
-    return set_error_msg(NBODY_ECUDA, "cudaEventCreate failed");
-  }
   int st = NBODY_OK;
-  bool ev_fail = false;
   float best = -1.0f;
   int bt = -1, bj = 0;
   std::vector<float> ts(static_cast<size_t>(reps));
@@ -125,19 +147,11 @@ int nbody_tune(int32_t table, const void *pos_m, const void *prm, int64_t n, flo
       }
       if (js == 0 && tiles[t].tile_i > 4 * n) continue;       // far more targets than particles
       st = run_once(table, pos_m, prm, n, eps2, t, js, o0, o1, om, s);  // warm-up
-      for (int r = 0; r < reps && st == NBODY_OK; ++r) {
-        ev_fail = cudaEventRecord(e0, s) != cudaSuccess;
-        if (!ev_fail) st = run_once(table, pos_m, prm, n, eps2, t, js, o0, o1, om, s);
-        if (!ev_fail && st == NBODY_OK)
-          ev_fail = cudaEventRecord(e1, s) != cudaSuccess ||
-                    cudaEventSynchronize(e1) != cudaSuccess ||
-                    cudaEventElapsedTime(&ts[size_t(r)], e0, e1) != cudaSuccess;
-        if (ev_fail) st = NBODY_ECUDA;
-      }
+      float med = 0.0f;
+      if (st == NBODY_OK) st = time_call(reps, ts, &med, s, [&]() {
+        return run_once(table, pos_m, prm, n, eps2, t, js, o0, o1, om, s);
+      });
       if (st != NBODY_OK) break;
-      std::vector<float> sorted(ts);
-      std::nth_element(sorted.begin(), sorted.begin() + reps / 2, sorted.end());
-      const float med = sorted[size_t(reps / 2)];
       if (best < 0.0f || med < best) {
         best = med;
         bt = t;
@@ -145,15 +159,27 @@ int nbody_tune(int32_t table, const void *pos_m, const void *prm, int64_t n, flo
       }
     }
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  if (ev_fail) return set_error_msg(NBODY_ECUDA, "timing events failed");
   if (st != NBODY_OK) return st;
   NB_TRY(sync_and_check(s));
   if (bt < 0) return set_error_msg(NBODY_EINVAL, "no tile fits n = %lld", (long long)n);
   int lg = 0;
   while ((int64_t(1) << (lg + 1)) <= n && lg < 62) ++lg;
-  NB_TRY(set_tuned(table, lg, bt, bj));
+  // Install the winner; where the streamed kernel that a default call would run is
+  // faster still, as a stored entry, which leaves such calls with it.
+  int old_tile = -1, old_js = 0;
+  bool old_caller = false;
+  tuned_entry(table, lg, &old_tile, &old_js, &old_caller);
+  NB_TRY(set_tuned(table, lg, bt, bj, false));
+  st = run_once(table, pos_m, prm, n, eps2, -1, 0, o0, o1, om, s);
+  float lib_ms = -1.0f;
+  if (st == NBODY_OK) st = time_call(reps, ts, &lib_ms, s, [&]() {
+    return run_once(table, pos_m, prm, n, eps2, -1, 0, o0, o1, om, s);
+  });
+  if (st != NBODY_OK) {
+    set_tuned(table, lg, old_tile, old_js, old_caller);
+    return st;
+  }
+  if (lib_ms > best) NB_TRY(set_tuned(table, lg, bt, bj, true));
   if (best_tile) *best_tile = bt;
   if (best_jsplit) *best_jsplit = bj;
   if (best_ms) *best_ms = best;

@@ -32,9 +32,86 @@ __device__ __forceinline__ void block_sum8(double v[kDiagFields], double *out) {
   }
 }
 
-__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const FinalizeArgs f) {
+// SPLIT 1: the partials of the tile kernels. SPLIT > 1: those of the streamed triangle
+// kernels; SPLIT threads share one particle's slots, each adding one of SPLIT equal
+// runs of them, and the first then adds the runs in order (at small n the finalize is
+// bound by the latency of one thread's loads: about 30 slots per particle at 8192
+// atoms, eight in flight).
+template <int SPLIT>
+__global__ void __launch_bounds__(kFinThreads * SPLIT) finalize_kernel(
+    const __grid_constant__ FinalizeArgs f) {
+  const int run_of = SPLIT > 1 ? threadIdx.x / kFinThreads : 0;
+  const int i = blockIdx.x * kFinThreads + (threadIdx.x - run_of * kFinThreads);
+  int below = 0, k0 = 0, k1 = 0;  // this thread's run of the particle's slots
+  if (SPLIT > 1) {
+    griddep_launch();
+    const int row = min(i, f.n - 1) / (64 * f.tri.h);
+    int first, shares;
+    tri_row_shares(f.tri, row, first, shares);
+    below = row + 1;
+    k0 = (below + shares) * run_of / SPLIT;
+    k1 = (below + shares) * (run_of + 1) / SPLIT;
+  }
   griddep_start();
-  const int i = blockIdx.x * kFinThreads + threadIdx.x;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 hi = zero, lo = zero;
+  const bool plain = f.plain != 0;
+  auto add = [&](const float4 &h, const float4 &l) {
+    if (plain) {
+      hi.x = __fadd_rn(hi.x, h.x);
+      hi.y = __fadd_rn(hi.y, h.y);
+      hi.z = __fadd_rn(hi.z, h.z);
+      hi.w = __fadd_rn(hi.w, h.w);
+    } else {
+      comp_add(hi.x, lo.x, h.x);
+      comp_add(hi.y, lo.y, h.y);
+      comp_add(hi.z, lo.z, h.z);
+      comp_add(hi.w, lo.w, h.w);
+    }
+    lo.x = __fadd_rn(lo.x, l.x);
+    lo.y = __fadd_rn(lo.y, l.y);
+    lo.z = __fadd_rn(lo.z, l.z);
+    lo.w = __fadd_rn(lo.w, l.w);
+  };
+  // `count` slots k0, k0 + step, ...; loads issued eight slots ahead of the
+  // adds (the symmetric tiles leave one slot per block and source part: a
+  // hundred or more per particle, read by few CTAs at small N)
+  auto run = [&](int k0, int count, int step) {
+    constexpr int U = 8;
+    int c = 0;
+    for (; c + U <= count; c += U) {
+      float4 h[U], l[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const long long o = (long long)(k0 + (c + u) * step) * f.stride + i;
+        h[u] = f.part_hi[o];
+        l[u] = f.part_lo ? f.part_lo[o] : zero;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) add(h[u], l[u]);
+    }
+    for (; c < count; ++c) {
+      const long long o = (long long)(k0 + c * step) * f.stride + i;
+      add(f.part_hi[o], f.part_lo ? f.part_lo[o] : zero);
+    }
+  };
+  if constexpr (SPLIT > 1) {
+    __shared__ float4 runs[2][SPLIT - 1][kFinThreads];
+    if (i < f.n) {
+      // the source-side slots 0 .. row, then the target-side slots from nb on
+      run(k0, min(k1, below) - k0, 1);
+      run(f.tri.nb + max(k0, below) - below, k1 - max(k0, below), 1);
+    }
+    const int at = threadIdx.x - run_of * kFinThreads;
+    if (run_of > 0) {
+      runs[0][run_of - 1][at] = hi;
+      runs[1][run_of - 1][at] = lo;
+    }
+    __syncthreads();
+    if (run_of > 0) return;
+#pragma unroll
+    for (int q = 0; q < SPLIT - 1; ++q) add(runs[0][q][at], runs[1][q][at]);
+  }
   double dv[kDiagFields] = {0, 0, 0, 0, 0, 0, 0, 0};
   float4 xn = make_float4(1e18f, 1e18f, 1e18f, 0.0f);  // drifted position (pad: far away)
   if (i < f.n) {
@@ -103,50 +180,10 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(const FinalizeArg
                         float(dz - double(t.z)), float(dw - double(t.w)));
       } else {
         // part_lo == nullptr: partials without low parts (symmetric tiles)
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 hi = zero, lo = zero;
-        const bool plain = f.plain != 0;
-        auto add = [&](const float4 &h, const float4 &l) {
-          if (plain) {
-            hi.x = __fadd_rn(hi.x, h.x);
-            hi.y = __fadd_rn(hi.y, h.y);
-            hi.z = __fadd_rn(hi.z, h.z);
-            hi.w = __fadd_rn(hi.w, h.w);
-          } else {
-            comp_add(hi.x, lo.x, h.x);
-            comp_add(hi.y, lo.y, h.y);
-            comp_add(hi.z, lo.z, h.z);
-            comp_add(hi.w, lo.w, h.w);
-          }
-          lo.x = __fadd_rn(lo.x, l.x);
-          lo.y = __fadd_rn(lo.y, l.y);
-          lo.z = __fadd_rn(lo.z, l.z);
-          lo.w = __fadd_rn(lo.w, l.w);
-        };
-        // `count` slots k0, k0 + step, ...; loads issued eight slots ahead of the
-        // adds (the symmetric tiles leave one slot per block and source part: a
-        // hundred or more per particle, read by few CTAs at small N)
-        auto run = [&](int k0, int count, int step) {
-          constexpr int U = 8;
-          int c = 0;
-          for (; c + U <= count; c += U) {
-            float4 h[U], l[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-              const long long o = (long long)(k0 + (c + u) * step) * f.stride + i;
-              h[u] = f.part_hi[o];
-              l[u] = f.part_lo ? f.part_lo[o] : zero;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) add(h[u], l[u]);
-          }
-          for (; c < count; ++c) {
-            const long long o = (long long)(k0 + c * step) * f.stride + i;
-            add(f.part_hi[o], f.part_lo ? f.part_lo[o] : zero);
-          }
-        };
-        run(own_s, own_b, sp);
-        run(k_all, slices - k_all, 1);
+        if (SPLIT == 1) {
+          run(own_s, own_b, sp);
+          run(k_all, slices - k_all, 1);
+        }
         // Round hi + lo to FP32 and keep the residual (Fast2Sum, |hi| >= |lo|).
         t.x = __fadd_rn(hi.x, lo.x);
         r.x = __fsub_rn(lo.x, __fsub_rn(t.x, hi.x));

@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include "tri_plan.h"
+
 namespace nbody {
 
 // Per-system data of a batched run (one entry per system).
@@ -63,6 +65,10 @@ struct FinalizeArgs {
   int jn_block;
   int jn_words;
   int rezero;  // atomic plans: zero the accumulators after reading them
+  // Streamed triangle kernels (tri_plan.h): particle i of row b counts the slots
+  // 0 .. b (source side) and nb .. nb + (shares of row b) - 1 (target side).
+  // tri.h == 0: another kernel's slots.
+  TriGeom tri;
   // With kFinDiag: also add the block rows of diag_part into diag_out (8 doubles)
   // in the last block to finish, which diag_ticket (zero before the launch, zero
   // again after it) elects; null: only the block rows are written.
@@ -71,6 +77,7 @@ struct FinalizeArgs {
 };
 
 constexpr int kFinThreads = 64;  // many CTAs: the finalize is latency-bound at small n
+constexpr int kFinSplit = 4;     // threads that share a particle's slots (streamed kernels)
 constexpr int kDiagFields = 8;  // K, U, Px, Py, Pz, Lx, Ly, Lz
 
 }  // namespace nbody

@@ -109,12 +109,21 @@ __device__ __forceinline__ float rsqrt_newton(float y, float s) {
 // Programmatic dependent launch: returns once the grid this one depends on has
 // completed and its writes are visible (a no-op for a grid launched without the
 // programmatic-serialization attribute). Called first thing by every kernel of
-// the force / step chain, before it touches global memory. No kernel triggers
-// its dependents early: the next grid is launched as this one's last CTAs exit,
-// so its CTAs are placed on an idle GPU (placed while the previous grid still
-// held the SMs, the CTAs of a grid under one wave bunch up on a few SMs).
+// the force / step chain, before it touches global memory.
 __device__ __forceinline__ void griddep_start() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Programmatic dependent launch: lets the next grid of the chain be placed before
+// this one ends; what that grid reads of this one's writes it reads after its own
+// griddep_start. Called by the streamed triangle kernels, whose grid fills every SM to
+// the last register (whatever is placed early waits for a whole CTA to leave), and by
+// the finalize in front of them. The other kernels do not call it: their next grid is
+// launched as their last CTAs exit, so that its CTAs are placed on an idle GPU (placed
+// while the previous grid still held the SMs, the CTAs of a grid under one wave bunch
+// up on a few SMs).
+__device__ __forceinline__ void griddep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Knuth's TwoSum: s + e == a + b exactly, s = fl(a + b).

@@ -19,7 +19,7 @@ import numpy as np
 
 from . import api
 from ._lib import (LAW_GRAV, LAW_LJC, LAW_LJC_LINEAR, TABLE_BATCHED, TABLE_GRAV_FIXED,
-                   TABLE_JERK, TABLE_VJP_GRAV, TABLE_VJP_LJC, TABLE_VJP_LJC_LINEAR)
+                   TABLE_JERK, TABLE_VJP_GRAV, TABLE_VJP_LJC, TABLE_VJP_LJC_LINEAR, check, load)
 
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuned.json")
 
@@ -220,7 +220,8 @@ def load_cache(path: str = CACHE) -> int:
     count = 0
     for law, table in data.items():
         for bucket, ent in table.items():
-            api.set_tuned(int(law), 2 ** int(bucket), int(ent["tile"]), int(ent["jsplit"]))
+            check(load().nbody_set_stored(int(law), int(bucket), int(ent["tile"]),
+                                          int(ent["jsplit"])), "nbody_set_stored")
             count += 1
     return count
 
