@@ -112,7 +112,7 @@ struct ScratchSizes {
 ScratchSizes scratch_sizes(int law, int n, const Plan1 &plan, int diag_rows) {
   ScratchSizes z{};
   // FX: int64 (z, w)
-  const bool lo = !plan.atomic && !plan.tri && (!plan.tile->sym || plan.tile->fixed);
+  const bool lo = plan.direct || (!plan.atomic && !plan.tri && (!plan.tile->sym || plan.tile->fixed));
   const int64_t jn = plan.tile->sym ? int64_t(plan.slices) * plan.slice_len : n;
   z.part = plan.atomic ? round_up(size_t(8) * size_t(n) * sizeof(long long), 256)
                        : round_up(size_t(plan.slices) * size_t(n) * sizeof(float4), 256);
@@ -120,7 +120,7 @@ ScratchSizes scratch_sizes(int law, int n, const Plan1 &plan, int diag_rows) {
   const int nblk = std::max(1, (n + kFinThreads - 1) / kFinThreads);
   z.dpart = round_up(size_t(nblk) * kDiagFields * sizeof(double), 256);
   z.drows = round_up(size_t(std::max(diag_rows, 1)) * kDiagFields * sizeof(double), 256);
-  z.jb = plan.tri ? 0 : jbuf_bytes(law, jn);
+  z.jb = plan.tri ? 0 : plan.direct ? round_up(size_t(n) * sizeof(float4), 256) : jbuf_bytes(law, jn);
   z.msum = plan.atomic ? round_up(size_t((n + 511) / 512) * sizeof(double), 256) : 0;
   return z;
 }
@@ -207,12 +207,31 @@ int prepare_fixed(const float4 *pos, int n, const nbody_params &p, const Plan1 &
   return NBODY_OK;
 }
 
+int direct_args(const float4 *pos, const float4 *prm, float4 *acc, int n, const nbody_params &p,
+                DirectArgs *d) {
+  d->pos = pos;
+  d->prm = prm;
+  d->n_t = n;
+  d->n = n;
+  d->eps2 = p.eps2;
+  d->G = p.G;
+  d->law = p.law;
+  d->mode = kFinWriteAcc;
+  d->acc = acc;
+  return error_word(&d->err);
+}
+
 int forces_device(const float4 *pos, const float4 *prm, float4 *acc, float4 *acc_lo, int n,
                   const nbody_params &p, int sms, cudaStream_t s) {
   Plan1 plan{};
   NB_TRY(plan_single(table_of(p), n, p.tile, p.jsplit, sms, &plan, true, atomic_ok(p)));
   Scratch sc{};
   NB_TRY(get_scratch(s, p.law, n, plan, 0, &sc));
+  if (plan.direct && !acc_lo && !overlaps(acc, n, pos, n) && !(prm && overlaps(acc, n, prm, n))) {
+    DirectArgs d{};
+    NB_TRY(direct_args(pos, prm, acc, n, p, &d));
+    return launch_direct(d, plan.dplan, p.flags, (p.flags & NBODY_COMPUTE_POT) != 0, s);
+  }
   NB_TRY(prepare_fixed(pos, n, p, plan, sc, s));
   int *err = nullptr;
   NB_TRY(error_word(&err));
@@ -225,6 +244,70 @@ int forces_device(const float4 *pos, const float4 *prm, float4 *acc, float4 *acc
                            s, nullptr, true);
 }
 
+// Leapfrog steps as direct launches, one per force evaluation: each computes the
+// acceleration of its targets, kicks them and writes their drifted positions into the
+// other of two position buffers (the caller's, the scratch's), which the next one reads;
+// the last drift lands in the caller's. A reported evaluation is a direct launch and a
+// finalize, which sums the diagnostics and drifts in place.
+int step_direct(float4 *pos, float4 *vel, float4 *acc, const float4 *prm, int n, float dt,
+                int nsteps, int report_every, double *diag_dev, float4 *trace, float4 *state_lo,
+                const nbody_params &p, const Plan1 &plan, const Scratch &sc, cudaStream_t s) {
+  auto report = [&](int step) { return report_every > 0 && step % report_every == 0; };
+  auto trace_at = [&](int step) { return trace ? trace + size_t(step) * size_t(n) : nullptr; };
+  const bool want_pot = (p.flags & NBODY_COMPUTE_POT) != 0;
+  const bool eval0 = !(p.flags & NBODY_ACC_VALID) || report(0);
+  float4 *buf[2] = {pos, sc.jbuf};
+  int cur = 0;  // the buffer that holds the next evaluation's positions
+  for (int st = eval0 ? 0 : 1; st < nsteps; ++st) cur ^= report(st) ? 0 : 1;
+  DirectArgs d{};
+  NB_TRY(direct_args(pos, prm, acc, n, p, &d));
+  d.vel = vel;
+  d.dt = dt;
+  d.x_lo = state_lo;
+  d.v_lo = state_lo ? state_lo + n : nullptr;
+  FinalizeArgs f{};
+  f.vel = vel;
+  f.acc = acc;
+  f.dt = dt;
+  f.x_lo = d.x_lo;
+  f.v_lo = d.v_lo;
+  if (trace) NB_CUDA(cudaMemcpyAsync(trace, pos, size_t(n) * sizeof(float4),
+                                     cudaMemcpyDeviceToDevice, s));
+  if (!eval0) {  // first half-kick and drift from the caller's acceleration
+    kick_drift_to_kernel<<<(n + 127) / 128, 128, 0, s>>>(pos, vel, acc, n, dt, buf[cur],
+                                                         trace_at(1), d.x_lo, d.v_lo);
+    NB_CUDA(cudaGetLastError());
+    d.pdl = 1;
+  } else if (cur) {
+    NB_CUDA(cudaMemcpyAsync(buf[1], pos, size_t(n) * sizeof(float4), cudaMemcpyDeviceToDevice, s));
+  }
+  int row = 0;
+  for (int st = eval0 ? 0 : 1; st <= nsteps; ++st) {
+    const bool last = st == nsteps;
+    const int mode = kFinWriteAcc | (st > 0 ? kFinKickSync : 0) | (last ? 0 : kFinKickDrift);
+    if (report(st)) {
+      f.pos = buf[cur];
+      f.mode = mode | kFinDiag;
+      f.trace_next = last ? nullptr : trace_at(st + 1);
+      f.diag_out = sc.diag_rows + kDiagFields * row++;
+      NB_TRY(eval_and_finalize(buf[cur], prm, p, n, plan, sc, d.err, true, f, s, nullptr, false,
+                               false, false, nullptr, nullptr, d.pdl != 0));
+    } else {
+      d.pos = buf[cur];
+      d.pos_out = buf[cur ^ 1];
+      d.trace = last ? nullptr : trace_at(st + 1);
+      d.mode = mode;
+      NB_TRY(launch_direct(d, plan.dplan, p.flags, last && want_pot, s));
+      cur ^= 1;
+    }
+    d.pdl = 1;
+  }
+  if (row > 0)
+    NB_CUDA(cudaMemcpyAsync(diag_dev, sc.diag_rows, size_t(row) * kDiagFields * sizeof(double),
+                            cudaMemcpyDefault, s));
+  return NBODY_OK;
+}
+
 int step_device(float4 *pos, float4 *vel, float4 *acc, const float4 *prm, int n, float dt,
                 int nsteps, int report_every, double *diag_dev, float4 *trace, float4 *state_lo,
                 const nbody_params &p, int sms, cudaStream_t s) {
@@ -233,6 +316,9 @@ int step_device(float4 *pos, float4 *vel, float4 *acc, const float4 *prm, int n,
   const int rows = report_every > 0 ? nsteps / report_every + 1 : 0;
   Scratch sc{};
   NB_TRY(get_scratch(s, p.law, n, plan, rows, &sc));
+  if (plan.direct && nsteps > 0)
+    return step_direct(pos, vel, acc, prm, n, dt, nsteps, report_every, diag_dev, trace, state_lo,
+                       p, plan, sc, s);
   NB_TRY(prepare_fixed(pos, n, p, plan, sc, s));
   int *err = nullptr;
   NB_TRY(error_word(&err));

@@ -372,12 +372,51 @@ bool sym_fits(int64_t n, int block) {
 
 bool sym_atomic_law(int law) { return law == NBODY_LAW_GRAV || law == kTableGravFixed; }
 
+int launch_direct(const DirectArgs &a, const DirectPlan &plan, uint32_t flags, bool pot,
+                  cudaStream_t s, bool timed) {
+  const DirectLauncher go = a.law == NBODY_LAW_GRAV  ? direct_grav
+                            : a.law == NBODY_LAW_LJC ? direct_ljc
+                                                     : direct_ljclin;
+  DirectArgs d = a;
+  d.slices = plan.slices;
+  // 16 targets' gravity with potentials leave one CTA on an SM: 8 (the same sums: their
+  // order depends on the slices alone)
+  const bool big = plan.big && !(a.law == NBODY_LAW_GRAV && pot);
+  const TimerMark tm = timed ? timer_begin(0, s) : TimerMark{};
+  const cudaError_t e = go(d, big, pot, (flags & NBODY_PRECISE_RSQRT) != 0, s);
+  timer_end(tm, s);
+  if (e != cudaSuccess)
+    return set_error_msg(e == cudaErrorNoKernelImageForDevice ? NBODY_EUNSUPPORTED : NBODY_ECUDA,
+                         "force kernel launch failed: %s", cudaGetErrorString(e));
+  return NBODY_OK;
+}
+
+namespace {
+// What a plan without a tile names as its tile: none of a table, reads the positions
+// directly.
+const TileDesc kNoTile{};
+}  // namespace
+
+bool plan_direct(int law, int64_t n, int sms, Plan1 *out) {
+  if (law < 0 || law > NBODY_LAW_LJC_LINEAR || n < 1 || !direct_all(law, n, sms) ||
+      tuned_by_caller(law, n) || !direct_plan(law, false, n, n, sms, &out->dplan))
+    return false;
+  out->tile = &kNoTile;
+  out->tri = nullptr;
+  out->direct = true;
+  out->slices = 1;
+  out->slice_len = int(n);
+  out->n_itiles = 1;
+  out->grid = 1;
+  out->sym_split = 1;
+  out->atomic = false;
+  return true;
+}
+
 bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out) {
-  // Below about 2500 particles a row or two of targets cannot fill the GPU and the
-  // finalize is a launch more than the one-sided tiles' work is worth (steps at 2048:
-  // gravity 11.2 us against 9.0, LJC 11.0 both; at 4001: 15.7 against 21.7, 18.1
-  // against 30.5).
-  if (law < 0 || law > NBODY_LAW_LJC_LINEAR || n < 2500 || n > 0x7fffffffLL - 64 * 64 ||
+  // Below (and up to twice that for gravity) the direct kernels run: a row or two of
+  // targets cannot fill the GPU, and the finalize is a launch more.
+  if (law < 0 || law > NBODY_LAW_LJC_LINEAR || n < 2048 || n > 0x7fffffffLL - 64 * 64 ||
       tuned_by_caller(law, n))
     return false;
   const TriDesc *d = law == NBODY_LAW_GRAV ? tri_grav(n)
@@ -392,10 +431,9 @@ bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out) {
   // against 17.8), where the slots would grow as n^2 (134 MB and 2.1 GB).
   if (law == NBODY_LAW_GRAV && atomic_ok && n >= 65536) return false;
   if (bytes > sym_part_cap()) return false;
-  // The plan's tile: none of a table, reads the positions directly.
-  static const TileDesc direct{};
-  out->tile = &direct;
+  out->tile = &kNoTile;
   out->tri = d;
+  out->direct = false;
   out->geom = g;
   out->slices = slots;
   out->slice_len = 0;
@@ -408,7 +446,8 @@ bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out) {
 
 int plan_single(int law, int64_t n, int tile, int jsplit, int sms, Plan1 *out, bool allow_sym,
                 bool atomic_ok) {
-  if (tile < 0 && jsplit <= 0 && allow_sym && plan_tri(law, n, sms, atomic_ok, out))
+  if (tile < 0 && jsplit <= 0 && allow_sym &&
+      (plan_direct(law, n, sms, out) || plan_tri(law, n, sms, atomic_ok, out)))
     return NBODY_OK;
   return plan_targets(law, n, n, tile, jsplit, sms, out, allow_sym, atomic_ok);
 }
@@ -417,6 +456,7 @@ int plan_targets(int law, int64_t n_t, int64_t n, int tile, int jsplit, int sms,
                  bool allow_sym, bool atomic_ok) {
   out->atomic = false;
   out->tri = nullptr;
+  out->direct = false;
   if (law < 0 || law >= kTableVjpGrav)
     return set_error_msg(NBODY_EINVAL, "tile table %d is not a force table", law);
   int count = 0;
@@ -640,6 +680,21 @@ int launch_forces(const float4 *pos, const float4 *prm, int law, uint32_t flags,
                                         !at->ticket || !at->scale || !at->inv)))
     return set_error_msg(NBODY_EINVAL, "atomic plan and accumulators must come together");
   if (atomic) fscale = at->scale;
+  if (p.direct) {  // the sums alone; direct steps launch with their epilogue themselves
+    if (tg || kd || atomic)
+      return set_error_msg(NBODY_EINVAL, "the direct kernels take all targets as they are");
+    DirectArgs d{};
+    d.pos = pos;
+    d.prm = prm;
+    d.n_t = d.n = n;
+    d.eps2 = eps2;
+    d.law = law;
+    d.err = err;
+    d.acc = part_hi;
+    d.acc_lo = part_lo;
+    d.pdl = chained ? 1 : 0;
+    return launch_direct(d, p.dplan, flags, pot, s, timed);
+  }
   if (p.tri) {  // streamed triangle kernel: reads pos / prm themselves
     if (tg || kd || atomic)
       return set_error_msg(NBODY_EINVAL, "the streamed kernels take all targets as they are");

@@ -15,6 +15,7 @@
 
 #include "nbody.h"
 #include "tiles.h"
+#include "direct_tiles.h"
 #include "tri_tiles.h"
 
 namespace nbody {
@@ -93,6 +94,8 @@ struct Plan1 {
   int sym_split;   // symmetric tiles: source parts per block (1 otherwise)
   const TriDesc *tri;  // streamed triangle kernel (tri_kernel.cuh) instead of the tile,
   TriGeom geom;        // its shares (`slices` is then its slot count), or null
+  bool direct;         // direct kernel (direct_kernel.cuh) instead of the tile: one slot
+  DirectPlan dplan;
   bool atomic;     // symmetric gravity: per-block partials added with integer atomics
                    // into fixed-point accumulators per particle (scratch 64 bytes
                    // per particle) instead of one slot per block
@@ -118,6 +121,19 @@ int plan_targets(int law, int64_t n_t, int64_t n, int tile, int jsplit, int sms,
 // library, or false where a tile runs: an entry of the tile table that the caller
 // installed (nbody_set_tuned, nbody_tune), or a partial-sum buffer above its limit.
 bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out);
+// Whether two float4 arrays share memory (a direct launch writes accelerations while
+// other CTAs still read positions).
+inline bool overlaps(const void *a, int64_t na, const void *b, int64_t nb) {
+  const auto x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + uintptr_t(nb) * 16 && y < x + uintptr_t(na) * 16;
+}
+// One direct launch (direct_kernel.cuh) for a law, `timed` like the other force kernels.
+int launch_direct(const DirectArgs &a, const DirectPlan &plan, uint32_t flags, bool pot,
+                  cudaStream_t s, bool timed = true);
+// Plan of a direct launch for all n particles of a call that leaves the configuration to
+// the library, or false where another kernel runs (a larger system, an entry of the tile
+// table that the caller installed).
+bool plan_direct(int law, int64_t n, int sms, Plan1 *out);
 // Whether the symmetric tiles of tile table `law` can accumulate atomically
 // (gravity and fixed-point gravity).
 bool sym_atomic_law(int law);

@@ -66,6 +66,26 @@ extern "C" int nbody_forces_subset(const void *pos_m, const void *prm, const int
     if (q && is_host_pointer(q)) return set_error_msg(NBODY_EINVAL, "device pointers only");
 
   const int nt = int(n_active), ns = int(n);
+  DirectPlan direct{};
+  if (p.tile < 0 && p.jsplit == 0 && !tuned_by_caller(p.law, nt) &&
+      !overlaps(acc, nt, pos_m, n) && !(prm && overlaps(acc, nt, prm, n)) &&
+      !overlaps(acc, nt, idx, (n_active + 3) / 4) &&
+      direct_plan(p.law, (p.flags & NBODY_COMPUTE_POT) != 0, nt, ns, sms, &direct)) {
+    DirectArgs d{};
+    d.pos = static_cast<const float4 *>(pos_m);
+    d.prm = static_cast<const float4 *>(prm);
+    d.idx = idx;
+    d.n_t = nt;
+    d.n = ns;
+    NB_TRY(error_word(&d.err));
+    d.eps2 = p.eps2;
+    d.G = p.G;
+    d.law = p.law;
+    d.mode = kFinWriteAcc;
+    d.acc = static_cast<float4 *>(acc);
+    return launch_direct(d, direct, p.flags, (p.flags & NBODY_COMPUTE_POT) != 0,
+                         reinterpret_cast<cudaStream_t>(stream));
+  }
   Plan1 plan{};
   NB_TRY(plan_targets(p.law, nt, ns, p.tile, p.jsplit, sms, &plan));
   const size_t jb = jbuf_bytes(p.law, ns);

@@ -340,6 +340,16 @@ __global__ void kick_drift_kernel(float4 *pos, float4 *vel, const float4 *acc, i
   kick_drift_at(pos, vel, acc, dt, trace1, x_lo, v_lo, i);
 }
 
+// The same for direct steps (direct_kernel.cuh): the drifted positions go to x_out
+// (which may be pos).
+__global__ void kick_drift_to_kernel(const float4 *pos, float4 *vel, const float4 *acc, int n,
+                                     float dt, float4 *x_out, float4 *trace1, float4 *x_lo,
+                                     float4 *v_lo) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  x_out[i] = kick_drift_from(pos[i], vel, acc, dt, trace1, x_lo, v_lo, i);
+}
+
 // Packing: caller SoA doubles -> (x, y, z, m) float4.
 __global__ void pack_grav_kernel(const double *x, const double *y, const double *z,
                                  const double *m, float4 *out, long long n) {

@@ -1,0 +1,10 @@
+// direct_grav.cu -- one-launch forces on few targets: softened gravity (Eq. 1).
+#include "direct_impl.h"
+
+namespace nbody {
+
+cudaError_t direct_grav(const DirectArgs &a, bool big, bool pot, bool precise, cudaStream_t s) {
+  return direct_law<TriGrav, 4>(a, big, pot, precise, s);
+}
+
+}  // namespace nbody

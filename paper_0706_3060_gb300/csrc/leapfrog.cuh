@@ -22,13 +22,13 @@ __device__ __forceinline__ void comp_axpy(float4 &hi, float4 &lo, float c, const
   lo.z = e;
 }
 
-// First half-kick and drift of particle i from a known acceleration (leapfrog,
-// Sec. 2): v += dt/2 a, x += dt v, in place (with the two-float state when x_lo
-// is given); writes the drifted position to trace1 (if given) and returns it.
-__device__ __forceinline__ float4 kick_drift_at(float4 *pos, float4 *vel, const float4 *acc,
-                                                float dt, float4 *trace1, float4 *x_lo,
-                                                float4 *v_lo, int i) {
-  float4 x = pos[i], v = vel[i];
+// First half-kick and drift of particle i at x from a known acceleration (leapfrog,
+// Sec. 2): v += dt/2 a, x += dt v (with the two-float state when x_lo is given);
+// writes the drifted position to trace1 (if given) and returns it.
+__device__ __forceinline__ float4 kick_drift_from(float4 x, float4 *vel, const float4 *acc,
+                                                  float dt, float4 *trace1, float4 *x_lo,
+                                                  float4 *v_lo, int i) {
+  float4 v = vel[i];
   const float4 a = acc[i];
   const float h = 0.5f * dt;
   if (x_lo) {
@@ -46,10 +46,16 @@ __device__ __forceinline__ float4 kick_drift_at(float4 *pos, float4 *vel, const 
     x.y = fmaf(dt, v.y, x.y);
     x.z = fmaf(dt, v.z, x.z);
   }
-  pos[i] = x;
   vel[i] = v;
   if (trace1) trace1[i] = x;
   return x;
+}
+
+// The same in place.
+__device__ __forceinline__ float4 kick_drift_at(float4 *pos, float4 *vel, const float4 *acc,
+                                                float dt, float4 *trace1, float4 *x_lo,
+                                                float4 *v_lo, int i) {
+  return pos[i] = kick_drift_from(pos[i], vel, acc, dt, trace1, x_lo, v_lo, i);
 }
 
 }  // namespace nbody

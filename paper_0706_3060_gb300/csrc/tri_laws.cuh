@@ -5,12 +5,12 @@
 // A law gives the words of a particle (kWords: as a target two particles' words are
 // packed in float2, as a source they are broadcast to both halves), the number of
 // sums per particle (kSums) and the pair function
-//   pair<MASK>(S, T, A, J, e2, k0, k1, both)
+//   pair<MASK, SRC>(S, T, A, J, e2, k0, k1, both)
 // which adds the target-side terms of both targets to A and the source-side terms to
 // J (the even target's to J[2 c], the odd target's to J[2 c + 1]). MASK: a half counts
 // only when its k0 / k1 is set, and the source side only with `both`. kFlip bit c: the
 // source-side term of sum c has the opposite sign (Newton's third law), applied when J
-// is stored.
+// is stored. SRC false: the target side alone (direct_kernel.cuh).
 //
 // The source-side sums are plain floats updated with scalar fused multiply-adds: they
 // are added up and handed from lane to lane one word at a time (tri_kernel.cuh), and
@@ -70,7 +70,7 @@ struct TriGrav {
     w[1] = -w[1];
     w[2] = -w[2];
   }
-  template <bool MASK>
+  template <bool MASK, bool SRC = true>
   static __device__ __forceinline__ void pair(const float (&S)[kWords], const float2 (&T)[kWords],
                                               float2 (&A)[kSums], float (&J)[2 * kSums],
                                               float2 e2, bool k0 = true, bool k1 = true,
@@ -92,6 +92,7 @@ struct TriGrav {
     A[1] = __ffma2_rn(wi, dy, A[1]);
     A[2] = __ffma2_rn(wi, dz, A[2]);
     if (POT) A[kSums - 1] = __ffma2_rn(bcast(S[3]), y, A[kSums - 1]);
+    if (!SRC) return;
     float2 wj = __fmul2_rn(T[3], y3);  // target mass: pull on the source
     if (MASK) wj = only(wj, both);
     jfma(J, wj, dx);
@@ -124,7 +125,7 @@ struct TriLjc {
     w[1] = -w[1];
     w[2] = -w[2];
   }
-  template <bool MASK>
+  template <bool MASK, bool SRC = true>
   static __device__ __forceinline__ void pair(const float (&S)[kWords], const float2 (&T)[kWords],
                                               float2 (&A)[kSums], float (&J)[2 * kSums], float2,
                                               bool k0 = true, bool k1 = true,
@@ -153,15 +154,17 @@ struct TriLjc {
     A[0] = __ffma2_rn(f, dx, A[0]);
     A[1] = __ffma2_rn(f, dy, A[1]);
     A[2] = __ffma2_rn(f, dz, A[2]);
-    const float2 fj = MASK ? only(f, both) : f;
-    jfma(J, fj, dx);
-    jfma(J + 2, fj, dy);
-    jfma(J + 4, fj, dz);
+    if (SRC) {
+      const float2 fj = MASK ? only(f, both) : f;
+      jfma(J, fj, dx);
+      jfma(J + 2, fj, dy);
+      jfma(J + 4, fj, dz);
+    }
     if (POT) {
       float2 e = __fmul2_rn(qq, LIN ? y2 : y);
       e = __ffma2_rn(__fmul2_rn(ee, bcast(1.0f / 6.0f)), __ffma2_rn(u, u, neg2(u)), e);
       A[kSums - 1] = __fadd2_rn(A[kSums - 1], e);
-      jadd(J + 2 * (kSums - 1), MASK ? only(e, both) : e);
+      if (SRC) jadd(J + 2 * (kSums - 1), MASK ? only(e, both) : e);
     }
   }
 };
