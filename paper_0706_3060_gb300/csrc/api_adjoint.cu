@@ -34,6 +34,12 @@ struct VjpScratch {
   unsigned *ticket;
   float *fscale;
   double *finv;
+  unsigned *type_ticket;  // last-block ticket of the per-type sums (arena header)
+  // a kernel without a tile (d null): streamed triangle kernel and its shares, or
+  // (tri null) a direct launch
+  const TriDesc *tri;
+  TriGeom geom;
+  int table;
 };
 
 // When the symmetric gravity VJP (and, with the same params, acceleration + jerk)
@@ -56,6 +62,92 @@ int vjp_table(int law) {
   return law == NBODY_LAW_LJC ? kTableVjpLJC : kTableVjpGrav;
 }
 
+// A default call's kernel without a tile: up to one wave of direct CTAs (two of 8 targets
+// on every SM; 2432 particles on 152) a direct launch (direct_kernel.cuh), above the
+// streamed triangle kernel where its slots fit. Sets *planned and the scratch layout.
+// Per Hermite step, gravity and LJC reverse step (us), direct / streamed: 10.8, 11.8,
+// 22.8 / - at 2432, 14.3, 15.6, 26.4 / 16.0, 15.0, 26.0 at 2500, 17.9, 19.5, 36.9 at
+// 3500 against 21.8, 21.4, 37.1 at 4096.
+int vjp_untiled(int law, int n, int sms, cudaStream_t s, VjpScratch *sc, size_t extra,
+                bool *planned) {
+  const bool lj = law == NBODY_LAW_LJC || law == NBODY_LAW_LJC_LINEAR;
+  const int blocks = (lj || law == kLawGAJ) ? 2 : 1;
+  *planned = false;
+  int slots = 1;
+  if (n > 16 * sms) {
+    if (n > 0x7fffffff - 64 * 64) return NBODY_OK;
+    sc->tri = tri_vjp(sc->table);
+    sc->geom = tri_geom(n, sc->tri->h, sms * sc->tri->per_sm);
+    slots = sc->geom.nb + tri_max_row_shares(sc->geom);
+    if (double(blocks) * slots * n * sizeof(float4) > sym_part_cap()) {
+      sc->tri = nullptr;
+      return NBODY_OK;
+    }
+  }
+  const size_t part = round_up(size_t(blocks) * slots * size_t(n) * sizeof(float4), 256);
+  const size_t lo = sc->tri ? 0 : part;
+  const int per_block = sc->tri ? kSlotParts : 256;
+  sc->nblk = (n + per_block - 1) / per_block;
+  const size_t tbytes = round_up(size_t(sc->nblk) * 8 * sizeof(double), 256);
+  void *base = nullptr;
+  char *hdr = nullptr;
+  NB_TRY(workspace(s, part + lo + tbytes + extra, &base, &hdr));
+  char *b = static_cast<char *>(base);
+  sc->part_hi = reinterpret_cast<float4 *>(b);
+  sc->part_lo = lo ? reinterpret_cast<float4 *>(b + part) : nullptr;
+  sc->type_part = reinterpret_cast<double *>(b + part + lo);
+  sc->extra = b + part + lo + tbytes;
+  sc->type_ticket = reinterpret_cast<unsigned *>(hdr + 56);
+  sc->u = sc->jp = nullptr;
+  sc->acc64 = nullptr;
+  sc->vpart = nullptr;
+  sc->slices = slots;
+  sc->bstride = (long long)slots * n;
+  sc->d = nullptr;
+  sc->sym_split = 1;
+  *planned = true;
+  return NBODY_OK;
+}
+
+// The untiled kernel of sc: partial sums for the finalize.
+int launch_untiled(const float4 *pos, const float4 *prm, const float4 *vec, int n,
+                   const nbody_params &p, const VjpScratch &sc, int timer, cudaStream_t s,
+                   bool chained) {
+  const TimerMark tm = timer_begin(timer, s);
+  cudaError_t e;
+  if (sc.tri) {
+    TriArgs t{};
+    t.p0 = pos;
+    t.p1 = prm;
+    t.p2 = vec;
+    t.part = sc.part_hi;
+    t.ostride = sc.bstride;
+    t.eps2 = p.eps2;
+    t.geom = sc.geom;
+    t.pdl = chained ? 1 : 0;
+    e = sc.tri->launch(t, false, false, s);
+  } else {
+    DirectArgs d{};
+    d.pos = pos;
+    d.prm = prm;
+    d.vec = vec;
+    d.n_t = d.n = n;
+    d.slices = 1;
+    d.eps2 = p.eps2;
+    d.acc = sc.part_hi;
+    d.acc_lo = sc.part_lo;
+    d.ostride = sc.bstride;
+    d.pdl = chained ? 1 : 0;
+    NB_TRY(error_word(&d.err));
+    e = direct_vjp(sc.table, d, s);
+  }
+  timer_end(tm, s);
+  if (e != cudaSuccess)
+    return set_error_msg(e == cudaErrorNoKernelImageForDevice ? NBODY_EUNSUPPORTED : NBODY_ECUDA,
+                         "VJP kernel launch failed: %s", cudaGetErrorString(e));
+  return NBODY_OK;
+}
+
 // Tile (params tile >= 0, else the tuned or default row of the law's table)
 // and j-split (params jsplit > 0, else the tuned one, else the split whose
 // items best fill whole waves of resident CTAs), then the scratch layout.
@@ -65,6 +157,13 @@ int vjp_table(int law) {
 int vjp_prepare(int law, int n, int tile, int jsplit, int sms, cudaStream_t s, VjpScratch *sc,
                 size_t extra = 0, int atomic_mode = 0) {
   const int table = vjp_table(law);
+  sc->table = table;
+  sc->tri = nullptr;
+  if (tile < 0 && jsplit <= 0 && atomic_mode < 2 && !tuned_by_caller(table, n)) {
+    bool planned = false;
+    NB_TRY(vjp_untiled(law, n, sms, s, sc, extra, &planned));
+    if (planned) return NBODY_OK;
+  }
   int count = 0;
   const VjpDesc *tiles = vjp_tiles(table, &count);
   int tj = 0;
@@ -115,6 +214,7 @@ int vjp_prepare(int law, int n, int tile, int jsplit, int sms, cudaStream_t s, V
     char *hdr = nullptr;
     NB_TRY(workspace(s, part + ubytes + tbytes + jbytes + vbytes + extra, &base, &hdr));
     char *b = static_cast<char *>(base);
+    sc->type_ticket = reinterpret_cast<unsigned *>(hdr + 56);
     sc->part_hi = reinterpret_cast<float4 *>(b);
     sc->part_lo = nullptr;
     sc->u = reinterpret_cast<float4 *>(b + part);
@@ -169,8 +269,10 @@ int vjp_prepare(int law, int n, int tile, int jsplit, int sms, cudaStream_t s, V
   const size_t jbytes =
       d.packed ? round_up(size_t((n + 1) / 2) * pair_f4 * sizeof(float4), 256) : 0;
   void *base = nullptr;
-  NB_TRY(workspace(s, 2 * part + ubytes + tbytes + jbytes + extra, &base));
+  char *hdr = nullptr;
+  NB_TRY(workspace(s, 2 * part + ubytes + tbytes + jbytes + extra, &base, &hdr));
   char *b = static_cast<char *>(base);
+  sc->type_ticket = reinterpret_cast<unsigned *>(hdr + 56);
   sc->extra = b + 2 * part + ubytes + tbytes + jbytes;
   sc->jp = d.packed ? reinterpret_cast<float4 *>(b + 2 * part + ubytes + tbytes) : nullptr;
   sc->part_hi = reinterpret_cast<float4 *>(b);
@@ -187,13 +289,11 @@ int vjp_prepare(int law, int n, int tile, int jsplit, int sms, cudaStream_t s, V
   return NBODY_OK;
 }
 
-// One VJP: all-pairs kernel + finalize (+ type reduction). chained: the previous
-// operation in `s` is a kernel of this library issued by the same call, so every
-// launch here may be a programmatic dependent launch (otherwise all but the first).
-int vjp_once(const float4 *pos, const float4 *prm, const float4 *lam, float4 *grad_x,
-             float *grad_m, double *grad_types, int ntypes, float alpha, int accumulate, int n,
-             const nbody_params &p, const VjpScratch &sc, float4 *lam_v, float dt_next,
-             cudaStream_t s, bool chained) {
+// The tile kernel of one VJP and what it needs before it; *lam_u: what it takes as lambda
+// (LJC: u = lam / m).
+int launch_vjp_tile(const float4 *pos, const float4 *prm, const float4 *lam, const float4 **lam_u,
+                    int n, const nbody_params &p, const VjpScratch &sc, cudaStream_t s,
+                    bool chained) {
   int *err = nullptr;
   NB_TRY(error_word(&err));
   const float4 *src = lam;
@@ -245,13 +345,30 @@ int vjp_once(const float4 *pos, const float4 *prm, const float4 *lam, float4 *gr
   timer_end(tm, s);
   if (e != cudaSuccess)
     return set_error_msg(NBODY_ECUDA, "VJP kernel launch failed: %s", cudaGetErrorString(e));
+  *lam_u = src;
+  return NBODY_OK;
+}
+
+// One VJP: all-pairs kernel + finalize. chained: the previous
+// operation in `s` is a kernel of this library issued by the same call, so every
+// launch here may be a programmatic dependent launch (otherwise all but the first).
+int vjp_once(const float4 *pos, const float4 *prm, const float4 *lam, float4 *grad_x,
+             float *grad_m, double *grad_types, int ntypes, float alpha, int accumulate, int n,
+             const nbody_params &p, const VjpScratch &sc, float4 *lam_v, float dt_next,
+             int type_ends, cudaStream_t s, bool chained) {
+  const float4 *src = lam;
+  const bool ljc = (p.law == NBODY_LAW_LJC || p.law == NBODY_LAW_LJC_LINEAR);
+  if (!sc.d)
+    NB_TRY(launch_untiled(pos, prm, lam, n, p, sc, 1, s, chained));
+  else
+    NB_TRY(launch_vjp_tile(pos, prm, lam, &src, n, p, sc, s, chained));
   VjpFinalizeArgs f{};
   f.part_hi = sc.part_hi;
   f.part_lo = sc.part_lo;
   f.stride = n;
   f.bstride = sc.bstride;
   f.slices = sc.slices;
-  f.sym_block = sc.d->sym ? sc.d->tile_i : 0;
+  f.sym_block = sc.d && sc.d->sym ? sc.d->tile_i : 0;
   f.sym_split = sc.sym_split;
   f.n = n;
   f.law = p.law;
@@ -269,10 +386,17 @@ int vjp_once(const float4 *pos, const float4 *prm, const float4 *lam, float4 *gr
   f.dt_next = dt_next;
   f.acc64 = sc.acc64;
   f.fx_inv = sc.acc64 ? sc.finv : nullptr;
-  NB_CUDA(launch_kernel(vjp_finalize_kernel, sc.nblk, 256, 0, s, true, f));
-  if (types)
-    NB_CUDA(launch_kernel(type_reduce_kernel, 1, 32, 0, s, true, sc.type_part, sc.nblk, ntypes,
-                          grad_types));
+  f.lam_is_u = sc.d ? 1 : 0;
+  f.ticket = sc.type_ticket;
+  f.grad_types = grad_types;
+  f.ntypes = ntypes;
+  f.type_ends = type_ends;
+  if (sc.tri) {
+    f.tri = sc.geom;
+    NB_CUDA(launch_kernel(vjp_finalize_kernel<4>, sc.nblk, 256, 0, s, true, f));
+  } else {
+    NB_CUDA(launch_kernel(vjp_finalize_kernel<1>, sc.nblk, 256, 0, s, true, f));
+  }
   return NBODY_OK;
 }
 
@@ -304,84 +428,74 @@ int check_dev_ptrs(std::initializer_list<const void *> ptrs) {
   return NBODY_OK;
 }
 
-// Hermite predictor: x_p = x + dt (v + dt (a/2 + dt j/6)), v_p = v + dt (a + dt j/2).
 __global__ void hermite_predict_kernel(const float4 *pos, const float4 *vel, const float4 *acc,
                                        const float4 *jerk, float dt, int n, float4 *xp,
                                        float4 *vp) {
+  griddep_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float4 x = pos[i], v = vel[i], a = acc[i], j = jerk[i];
-  const float h2 = 0.5f * dt, h6 = dt * (1.0f / 6.0f);
-  xp[i] = make_float4(fmaf(dt, fmaf(dt, fmaf(h6, j.x, 0.5f * a.x), v.x), x.x),
-                      fmaf(dt, fmaf(dt, fmaf(h6, j.y, 0.5f * a.y), v.y), x.y),
-                      fmaf(dt, fmaf(dt, fmaf(h6, j.z, 0.5f * a.z), v.z), x.z), x.w);
-  vp[i] = make_float4(fmaf(dt, fmaf(h2, j.x, a.x), v.x), fmaf(dt, fmaf(h2, j.y, a.y), v.y),
-                      fmaf(dt, fmaf(h2, j.z, a.z), v.z), 0.0f);
+  if (i < n) hermite_predict(pos[i], vel[i], acc[i], jerk[i], dt, xp[i], vp[i]);
 }
 
-// Hermite corrector (time-symmetric form):
-//   v1 = v + dt/2 (a + a1) + dt^2/12 (j - j1),  x1 = x + dt/2 (v + v1) + dt^2/12 (a - a1)
-__global__ void hermite_correct_kernel(float4 *pos, float4 *vel, float4 *acc, float4 *jerk,
-                                       const float4 *a1v, const float4 *j1v, float dt, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float4 x = pos[i], v = vel[i], a = acc[i], j = jerk[i], a1 = a1v[i], j1 = j1v[i];
-  const float h = 0.5f * dt, q = dt * dt * (1.0f / 12.0f);
-  float4 v1, x1;
-  v1.x = fmaf(q, j.x - j1.x, fmaf(h, a.x + a1.x, v.x));
-  v1.y = fmaf(q, j.y - j1.y, fmaf(h, a.y + a1.y, v.y));
-  v1.z = fmaf(q, j.z - j1.z, fmaf(h, a.z + a1.z, v.z));
-  v1.w = v.w;
-  x1.x = fmaf(q, a.x - a1.x, fmaf(h, v.x + v1.x, x.x));
-  x1.y = fmaf(q, a.y - a1.y, fmaf(h, v.y + v1.y, x.y));
-  x1.z = fmaf(q, a.z - a1.z, fmaf(h, v.z + v1.z, x.z));
-  x1.w = x.w;
-  pos[i] = x1;
-  vel[i] = v1;
-  acc[i] = a1;
-  jerk[i] = j1;
-}
-
-// Acceleration and jerk at (pos, vel) into (acc, jerk): GAJ kernel + finalize.
-int gaj_eval(const float4 *pos, const float4 *vel, float4 *acc, float4 *jerk, int n,
-             const nbody_params &p, const VjpScratch &sc, cudaStream_t s) {
+// Acceleration and jerk at (pos, vel): GAJ kernel, then the finalize that f describes
+// (where they go, the corrector and the next predictor). chained: a kernel of this call
+// precedes.
+int gaj_eval(const float4 *pos, const float4 *vel, GajFinalizeArgs f, int n,
+             const nbody_params &p, const VjpScratch &sc, cudaStream_t s, bool chained) {
   int *err = nullptr;
   NB_TRY(error_word(&err));
-  if (sc.d->packed) {  // (x, m) and velocities of source pairs, interleaved
-    const unsigned pblocks = unsigned(((n + 1) / 2 + 255) / 256);
-    if (sc.d->sym)
-      interleave_vjp_pairs_blocked_kernel<<<pblocks, 256, 0, s>>>(
-          pos, vel, sc.jp, n, sc.d->tile_i,
-          VjpAtomicPrep{sc.acc64, sc.vpart, sc.ticket, p.eps2, sc.fscale, sc.finv, 1, 16});
-    else
-      interleave_vjp_pairs_kernel<<<pblocks, 256, 0, s>>>(pos, vel, sc.jp, n);
-    NB_CUDA(cudaGetLastError());
+  if (!sc.d) {
+    NB_TRY(launch_untiled(pos, nullptr, vel, n, p, sc, 0, s, chained));
+  } else {
+    if (sc.d->packed) {  // (x, m) and velocities of source pairs, interleaved
+      const int pblocks = ((n + 1) / 2 + 255) / 256;
+      if (sc.d->sym)
+        NB_CUDA(launch_kernel(interleave_vjp_pairs_blocked_kernel, pblocks, 256, 0, s, chained,
+                              pos, vel, sc.jp, n, sc.d->tile_i,
+                              VjpAtomicPrep{sc.acc64, sc.vpart, sc.ticket, p.eps2, sc.fscale,
+                                            sc.finv, 1, 16}));
+      else
+        NB_CUDA(launch_kernel(interleave_vjp_pairs_kernel, pblocks, 256, 0, s, chained, pos, vel,
+                              sc.jp, n));
+      chained = true;
+    }
+    VjpArgs a{};
+    a.pos = pos;
+    a.lam = vel;
+    a.jpair = sc.jp;
+    a.part_hi = sc.part_hi;
+    a.part_lo = sc.part_lo;
+    a.stride = n;
+    a.bstride = sc.bstride;
+    a.err = err;
+    a.n = n;
+    a.slices = sc.slices;
+    a.slice_len = sc.slice_len;
+    a.eps2 = p.eps2;
+    a.comp = (p.flags & NBODY_NO_COMPENSATION) ? 0 : 1;
+    a.pdl = chained ? 1 : 0;
+    a.acc64 = sc.acc64;
+    a.fscale = sc.acc64 ? sc.fscale : nullptr;
+    const TimerMark tm = timer_begin(0, s);
+    cudaError_t e = sc.d->launch(a, sc.grid, s);
+    timer_end(tm, s);
+    if (e != cudaSuccess)
+      return set_error_msg(NBODY_ECUDA, "jerk kernel launch failed: %s", cudaGetErrorString(e));
   }
-  VjpArgs a{};
-  a.pos = pos;
-  a.lam = vel;
-  a.jpair = sc.jp;
-  a.part_hi = sc.part_hi;
-  a.part_lo = sc.part_lo;
-  a.stride = n;
-  a.bstride = sc.bstride;
-  a.err = err;
-  a.n = n;
-  a.slices = sc.slices;
-  a.slice_len = sc.slice_len;
-  a.eps2 = p.eps2;
-  a.comp = (p.flags & NBODY_NO_COMPENSATION) ? 0 : 1;
-  a.acc64 = sc.acc64;
-  a.fscale = sc.acc64 ? sc.fscale : nullptr;
-  const TimerMark tm = timer_begin(0, s);
-  cudaError_t e = sc.d->launch(a, sc.grid, s);
-  timer_end(tm, s);
-  if (e != cudaSuccess)
-    return set_error_msg(NBODY_ECUDA, "jerk kernel launch failed: %s", cudaGetErrorString(e));
-  gaj_finalize_kernel<<<unsigned((n + 255) / 256), 256, 0, s>>>(
-      sc.part_hi, sc.part_lo, n, sc.bstride, sc.slices, n, p.G, acc, jerk, sc.acc64,
-      sc.acc64 ? sc.finv : nullptr);
-  NB_CUDA(cudaGetLastError());
+  f.part_hi = sc.part_hi;
+  f.part_lo = sc.part_lo;
+  f.stride = n;
+  f.bstride = sc.bstride;
+  f.slices = sc.slices;
+  f.n = n;
+  f.G = p.G;
+  f.acc64 = sc.acc64;
+  f.inv = sc.acc64 ? sc.finv : nullptr;
+  if (sc.tri) {
+    f.tri = sc.geom;
+    NB_CUDA(launch_kernel(gaj_finalize_kernel<4>, sc.nblk, 256, 0, s, true, f));
+  } else {
+    NB_CUDA(launch_kernel(gaj_finalize_kernel<1>, (n + 255) / 256, 256, 0, s, true, f));
+  }
   return NBODY_OK;
 }
 
@@ -433,7 +547,8 @@ int nbody_adjoint(const void *pos_m, const void *prm, const void *lam, void *gra
   }
   return vjp_once(static_cast<const float4 *>(pos_m), static_cast<const float4 *>(prm),
                   static_cast<const float4 *>(lam), static_cast<float4 *>(grad_x), grad_m,
-                  grad_types, ntypes, alpha, acc, int(n), p, sc, nullptr, 0.0f, s, launched);
+                  grad_types, ntypes, alpha, acc, int(n), p, sc, nullptr, 0.0f,
+                  kTypeFirst | kTypeLast, s, launched);
 }
 
 int nbody_adjoint_leapfrog(const void *xs, const void *prm, int64_t n, int32_t k, float dt,
@@ -468,7 +583,8 @@ int nbody_adjoint_leapfrog(const void *xs, const void *prm, int64_t n, int32_t k
     const float w = (st == 0 && first) ? 0.5f * dt : dt;
     // lam_x += w J(x_st)^T lam_v, then (except after the last) lam_v += dt lam_x.
     NB_TRY(vjp_once(X + size_t(st) * size_t(n), q, lv, lx, grad_m, grad_types, ntypes, w, 1,
-                    int(n), p, sc, st > 0 ? lv : nullptr, dt, s, true));
+                    int(n), p, sc, st > 0 ? lv : nullptr, dt,
+                    (st == k - 1 ? kTypeFirst : 0) | (st == 0 ? kTypeLast : 0), s, true));
   }
   return NBODY_OK;
 }
@@ -491,8 +607,11 @@ int nbody_forces_jerk(const void *pos_m, const void *vel, void *acc, void *jerk,
   VjpScratch sc{};
   NB_TRY(vjp_prepare(kLawGAJ, int(n), params->tile, params->jsplit, sms, s, &sc, 0,
                      vjp_atomic_mode(*params)));
-  return gaj_eval(static_cast<const float4 *>(pos_m), static_cast<const float4 *>(vel),
-                  static_cast<float4 *>(acc), static_cast<float4 *>(jerk), int(n), *params, sc, s);
+  GajFinalizeArgs f{};
+  f.acc = static_cast<float4 *>(acc);
+  f.jerk = static_cast<float4 *>(jerk);
+  return gaj_eval(static_cast<const float4 *>(pos_m), static_cast<const float4 *>(vel), f, int(n),
+                  *params, sc, s, false);
 }
 
 int nbody_hermite_step(void *pos_m, void *vel, void *acc, void *jerk, int64_t n, float dt,
@@ -512,28 +631,34 @@ int nbody_hermite_step(void *pos_m, void *vel, void *acc, void *jerk, int64_t n,
   NB_TRY(check_device(&dev, &sms));
   NB_TRY(check_dev_ptrs({pos_m, vel, acc, jerk}));
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  // scratch: GAJ partials, then predicted (x, v) and the new (a, j)
+  // scratch: GAJ partials, then predicted (x, v)
   VjpScratch sc{};
   const size_t q = round_up(size_t(n) * sizeof(float4), 256);
-  NB_TRY(vjp_prepare(kLawGAJ, int(n), params->tile, params->jsplit, sms, s, &sc, 4 * q,
+  NB_TRY(vjp_prepare(kLawGAJ, int(n), params->tile, params->jsplit, sms, s, &sc, 2 * q,
                      vjp_atomic_mode(*params)));
   float4 *xp = reinterpret_cast<float4 *>(sc.extra);
   float4 *vp = reinterpret_cast<float4 *>(sc.extra + q);
-  float4 *a1 = reinterpret_cast<float4 *>(sc.extra + 2 * q);
-  float4 *j1 = reinterpret_cast<float4 *>(sc.extra + 3 * q);
   float4 *X = static_cast<float4 *>(pos_m);
   float4 *V = static_cast<float4 *>(vel);
-  float4 *A = static_cast<float4 *>(acc);
-  float4 *J = static_cast<float4 *>(jerk);
   const int nn = int(n);
-  if (!(params->flags & NBODY_ACC_VALID)) NB_TRY(gaj_eval(X, V, A, J, nn, *params, sc, s));
-  const unsigned blocks = unsigned((n + 255) / 256);
+  GajFinalizeArgs f{};
+  f.acc = static_cast<float4 *>(acc);
+  f.jerk = static_cast<float4 *>(jerk);
+  bool launched = false;
+  if (!(params->flags & NBODY_ACC_VALID)) {
+    NB_TRY(gaj_eval(X, V, f, nn, *params, sc, s, false));
+    launched = true;
+  }
+  if (nsteps == 0) return NBODY_OK;
+  NB_CUDA(launch_kernel(hermite_predict_kernel, (nn + 255) / 256, 256, 0, s, launched, X, V, f.acc,
+                        f.jerk, dt, nn, xp, vp));
+  f.pos = X;
+  f.vel = V;
+  f.dt = dt;
   for (int st = 0; st < nsteps; ++st) {
-    hermite_predict_kernel<<<blocks, 256, 0, s>>>(X, V, A, J, dt, nn, xp, vp);
-    NB_CUDA(cudaGetLastError());
-    NB_TRY(gaj_eval(xp, vp, a1, j1, nn, *params, sc, s));
-    hermite_correct_kernel<<<blocks, 256, 0, s>>>(X, V, A, J, a1, j1, dt, nn);
-    NB_CUDA(cudaGetLastError());
+    f.xp = st + 1 < nsteps ? xp : nullptr;
+    f.vp = st + 1 < nsteps ? vp : nullptr;
+    NB_TRY(gaj_eval(xp, vp, f, nn, *params, sc, s, true));
   }
   return NBODY_OK;
 }

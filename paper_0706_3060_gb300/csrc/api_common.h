@@ -109,6 +109,8 @@ int default_tile(int law, int64_t n);
 // nb (nb + 1) / 2 block pairs within the grid limit and nb x n float4 partials
 // (nb = ceil(n / block)) within an eighth of the device's memory, at most 16 GiB.
 bool sym_fits(int64_t n, int block);
+// That limit on partial sums in bytes.
+double sym_part_cap();
 // atomic_ok: a symmetric gravity tile may accumulate atomically in fixed point
 // (the caller has eps > 0 and does not ask for plain FP32 sums); such a plan has
 // no partial-sum cap, only the grid limit on block pairs.

@@ -99,6 +99,13 @@ __device__ __forceinline__ float rsqrt_hw(float s) {
   return y;
 }
 
+// Hardware reciprocal (MUFU.RCP).
+__device__ __forceinline__ float rcp_hw(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // One Newton-Raphson step for 1/sqrt(s): y <- y (3 - s y^2) / 2 (textbook).
 __device__ __forceinline__ float rsqrt_newton(float y, float s) {
   const float hs = -0.5f * s;

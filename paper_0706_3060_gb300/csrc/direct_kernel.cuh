@@ -35,6 +35,7 @@ constexpr int kDirectFold = 32;  // sources per register sum
 struct DirectArgs {
   const float4 *pos;  // sources (x, y, z, m)
   const float4 *prm;  // LJC parameters or null
+  const float4 *vec;  // velocities or lambda (jerk and VJP laws), else null
   const int *idx;     // targets (a subset's indices), or null: all particles
   int n_t;
   int n;
@@ -49,6 +50,7 @@ struct DirectArgs {
   float dt;
   float4 *acc;       // element per target
   float4 *acc_lo;
+  long long ostride; // mode 0, laws of more than four sums: elements to their second row
   float4 *vel;
   float4 *pos_out;   // drifted positions (not `pos`: other CTAs still read it)
   float4 *trace;     // drifted positions as well, or null
@@ -83,7 +85,7 @@ __global__ void __launch_bounds__(kDirectThreads,
         g = 0;
       }
     }
-    L::load(a.pos, a.prm, nullptr, g >= 0 ? g : a.n, a.n, w);
+    L::load(a.pos, a.prm, a.vec, g >= 0 ? g : a.n, a.n, w);
     L::as_target(w);
 #pragma unroll
     for (int c = 0; c < L::kWords; ++c) words[c][tid] = w[c];
@@ -111,7 +113,7 @@ __global__ void __launch_bounds__(kDirectThreads,
   float P[U][L::kWords];
 #pragma unroll
   for (int u = 0; u < U; ++u)
-    L::load(a.pos, a.prm, nullptr, min(b0 + u, b1) * kDirectThreads + tid, a.n, P[u]);
+    L::load(a.pos, a.prm, a.vec, min(b0 + u, b1) * kDirectThreads + tid, a.n, P[u]);
   for (int b = b0; b < b1; b += U) {
     // every kDirectFold sources the sums go to this thread's own words in shared memory:
     // a close pair's large pull is not rounded again with each of hundreds of sources
@@ -140,7 +142,7 @@ __global__ void __launch_bounds__(kDirectThreads,
                                         tidx[2 * r + 1] != j);
       }
       if (b + u + U < b1)
-        L::load(a.pos, a.prm, nullptr, j + U * kDirectThreads, a.n, P[u]);
+        L::load(a.pos, a.prm, a.vec, j + U * kDirectThreads, a.n, P[u]);
     }
   }
   if (b1 - b0 > kDirectFold) {
@@ -230,14 +232,19 @@ __global__ void __launch_bounds__(kDirectThreads,
   const int t = t0 + tid;
   if (tid >= TG || t >= a.n_t) return;
   const int g = tidx[tid];
-  auto row = [&](const float (&v)[V]) {
-    return make_float4(v[tid], v[TG + tid], v[2 * TG + tid],
-                       NS > 3 ? v[(NS - 1) * TG + tid] : 0.0f);
+  auto row = [&](const float (&v)[V], int c0) {
+    constexpr int kRow = NS == 6 ? 3 : NS < 4 ? NS : 4;  // sums in a row
+    return make_float4(v[c0 * TG + tid], v[(c0 + 1) * TG + tid], v[(c0 + 2) * TG + tid],
+                       kRow > 3 ? v[(c0 + 3) * TG + tid] : 0.0f);
   };
-  const float4 hi = row(sums[0]), lo = row(sums[1]);
+  const float4 hi = row(sums[0], 0), lo = row(sums[1], 0);
   if (!a.mode) {
     a.acc[t] = hi;
     a.acc_lo[t] = lo;
+    if constexpr (NS > 4) {
+      a.acc[t + a.ostride] = row(sums[0], NS / 2);
+      a.acc_lo[t + a.ostride] = row(sums[1], NS / 2);
+    }
     return;
   }
   float4 x = a.pos[g], ac;

@@ -33,37 +33,45 @@ struct DirectPlan {
 // 1500 targets of 65536 in 16s and 3 slices 51 us (8s and 3 slices 69, 16s and 4 slices
 // 57). False where a thread's sum would have more than 32 folds at the most slices (n
 // above two million).
-inline bool direct_plan(int law, bool pot, int64_t n_t, int64_t n, int sms, DirectPlan *out) {
+struct DirectCost {
+  double block, fixed, alone, launch;  // us
+  bool one;                            // one CTA on an SM
+};
+// The least time over the slices (added to *out with `big` if less than *best).
+inline void direct_slices(const DirectCost &c, bool big, int64_t targets_per_cta, int64_t n_t,
+                          int64_t n, int sms, double *best, DirectPlan *out) {
   constexpr int64_t kChain = 32 * kDirectFold;
   static constexpr int kTwo[8] = {304, 304, 291, 296, 290, 276, 266, 288};
   static constexpr int kOne[8] = {152, 152, 138, 144, 140, 138, 105, 120};
-  struct Cost {
-    double block, fixed, alone, launch;  // us
-  };
-  static constexpr Cost kGrav[2] = {{0.296, 2.84, 0.66, 0.45}, {0.503, 3.06, 0.59, 0.61}};
-  static constexpr Cost kLjc[2] = {{0.533, 2.87, 0.76, 0.53}, {0.496, 3.24, 1.0, 0.57}};
-  if (n > kChain * kDirectThreads * 8 || n_t > (int64_t(1) << 28)) return false;
+  for (int s = 1; s <= 8; ++s) {
+    if (n > kChain * kDirectThreads * s) continue;
+    if (s > 1 && (s - 1) * kDirectThreads >= n) continue;  // an empty slice
+    const int64_t ctas = (n_t + targets_per_cta - 1) / targets_per_cta * s;
+    const int64_t held =
+        std::max<int64_t>(int64_t(c.one ? kOne[s - 1] : kTwo[s - 1]) * sms / 152, 1);
+    const int64_t waves = (ctas + held - 1) / held, last = ctas - (waves - 1) * held;
+    const double work = double((n + kDirectThreads * s - 1) / (kDirectThreads * s)) * c.block;
+    const double us = c.launch + (s > 1 ? 0.6 : 0.0) + double(waves) * c.fixed +
+                      work * (double(waves - 1) + (2 * last <= held ? c.alone : 1.0));
+    if (*best < 0.0 || us < *best) {
+      *best = us;
+      *out = DirectPlan{big, s};
+    }
+  }
+}
+inline bool direct_plan(int law, bool pot, int64_t n_t, int64_t n, int sms, DirectPlan *out) {
+  static constexpr DirectCost kGrav[2] = {{0.296, 2.84, 0.66, 0.45, false},
+                                          {0.503, 3.06, 0.59, 0.61, false}};
+  static constexpr DirectCost kLjc[2] = {{0.533, 2.87, 0.76, 0.53, false},
+                                         {0.496, 3.24, 1.0, 0.57, true}};
+  if (n_t > (int64_t(1) << 28)) return false;
   double best = -1.0;
   for (int big = 0; big < 2; ++big) {
     if (big && law == 0 && pot) continue;  // 16 targets' potentials leave one CTA on an SM
-    const Cost c = law == 0 ? kGrav[big] : kLjc[big];
-    for (int s = 1; s <= 8; ++s) {
-      if (n > kChain * kDirectThreads * s) continue;
-      if (s > 1 && (s - 1) * kDirectThreads >= n) continue;  // an empty slice
-      const int64_t tg = big ? 16 : 8, ctas = (n_t + tg - 1) / tg * s;
-      const int64_t held =
-          std::max<int64_t>(int64_t(big && law != 0 ? kOne[s - 1] : kTwo[s - 1]) * sms / 152, 1);
-      const int64_t waves = (ctas + held - 1) / held, last = ctas - (waves - 1) * held;
-      const double work = double((n + kDirectThreads * s - 1) / (kDirectThreads * s)) * c.block;
-      const double us = c.launch + (s > 1 ? 0.6 : 0.0) + double(waves) * c.fixed +
-                        work * (double(waves - 1) + (2 * last <= held ? c.alone : 1.0));
-      if (best < 0.0 || us < best) {
-        best = us;
-        *out = DirectPlan{big == 1, s};
-      }
-    }
+    direct_slices(law == 0 ? kGrav[big] : kLjc[big], big == 1, big ? 16 : 8, n_t, n, sms, &best,
+                  out);
   }
-  return true;
+  return best >= 0.0;
 }
 
 // Whether forces on all n particles run in one direct launch: one wave of two CTAs on
@@ -72,5 +80,9 @@ inline bool direct_plan(int law, bool pot, int64_t n_t, int64_t n, int sms, Dire
 // (us per step: gravity direct 13.1 at 4864, streamed 18.4 at 4865 where two direct waves
 // take 21; LJC direct 8.1 at 2432, 19.6 at 3000 where streamed takes 13.8).
 inline bool direct_all(int law, int64_t n, int sms) { return n <= (law == 0 ? 32 : 16) * sms; }
+
+// The jerk and VJP laws (tile tables of tri_vjp.cu): 8 targets per CTA, 4 for the LJC
+// VJPs; mode 0 only.
+cudaError_t direct_vjp(int table, const DirectArgs &a, cudaStream_t s);
 
 }  // namespace nbody

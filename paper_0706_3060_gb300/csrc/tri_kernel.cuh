@@ -53,8 +53,8 @@ constexpr int kTriLeft = 6;    // left-over groups of a window: three own, three
 
 struct TriArgs {
   const float4 *p0;  // (x, y, z, m)
-  const float4 *p1;  // LJC parameters, velocities, lambda or u (by law)
-  const float4 *p2;  // LJC VJP: the LJC parameters
+  const float4 *p1;  // LJC parameters
+  const float4 *p2;  // velocities, lambda, u (VJP and jerk laws)
   float4 *part;      // [slot][n], kSums floats each: one float4, or two (hi at ostride)
   long long ostride; // elements from the first float4 of a partial to its second
   float eps2;

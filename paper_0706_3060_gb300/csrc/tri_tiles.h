@@ -20,5 +20,7 @@ struct TriDesc {
 const TriDesc *tri_grav(int64_t n);
 const TriDesc *tri_ljc(int64_t n);
 const TriDesc *tri_ljclin(int64_t n);
+// Kernel for a VJP or jerk tile table (tri_vjp.cu; no potential or precise variants).
+const TriDesc *tri_vjp(int table);
 
 }  // namespace nbody

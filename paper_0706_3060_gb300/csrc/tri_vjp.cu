@@ -1,0 +1,53 @@
+// tri_vjp.cu -- streamed triangle and direct kernels of acceleration + jerk (Table 1
+// "Gravity (accel & jerk)") and of the gravity and LJC force VJPs.
+//
+// What bounds them: the packed FP32 unit (33, 35 and 64 operations per pair; 0.71, 0.72
+// and 0.78 of its rate at 32768), of which the three-operand multiply-adds take a sixth
+// more than the others. Rows of 256 targets: 226, 196 and 255 registers at two CTAs per
+// SM; rows of 384 spill (jerk: 642 us at 32768 against 614) or gain nothing (gravity VJP:
+// 637 against 642 at 32768, 165 against 166 at 16384, 48.0 against 46.4 at 8192), rows of
+// 128 move the sources twice as often (LJC VJP: 1153 us at 32768 against 1065).
+// Per step with the finalize, against the block-pair tiles (us):
+//   Hermite 8192 49.2 / 79.2, 16384 165 / 215, 32768 630 / 685
+//   gravity reverse step 4096 21.4 / 27.4, 8192 50.1 / 61.7, 16384 170 / 185
+//   LJC reverse step 4096 34.8 / 46.3, 8192 82 / 105, 32768 1097 / 2186
+#include "api_common.h"
+#include "direct_impl.h"
+#include "tri_impl.h"
+#include "tri_vjp_laws.cuh"
+
+namespace nbody {
+namespace {
+
+template <class L, int H, bool AHEAD>
+cudaError_t tri_one(const TriArgs &a, bool, bool, cudaStream_t s) {
+  return tri_go<L, H, 2, AHEAD>(a, s);
+}
+
+}  // namespace
+
+const TriDesc *tri_vjp(int table) {
+  static const TriDesc jerk{4, 2, &tri_one<TriJerk, 4, true>};
+  static const TriDesc grav{4, 2, &tri_one<TriGravVjp, 4, true>};
+  static const TriDesc ljc{4, 2, &tri_one<TriLjcVjp<false>, 4, true>};
+  static const TriDesc ljclin{4, 2, &tri_one<TriLjcVjp<true>, 4, true>};
+  switch (table) {
+    case kTableJerk: return &jerk;
+    case kTableVjpGrav: return &grav;
+    case kTableVjpLJC: return &ljc;
+    case kTableVjpLJCLin: return &ljclin;
+  }
+  return nullptr;
+}
+
+cudaError_t direct_vjp(int table, const DirectArgs &a, cudaStream_t s) {
+  switch (table) {
+    case kTableJerk: return direct_go<TriJerk, 4, 2>(a, s);
+    case kTableVjpGrav: return direct_go<TriGravVjp, 4, 2>(a, s);
+    case kTableVjpLJC: return direct_go<TriLjcVjp<false>, 2, 2>(a, s);
+    case kTableVjpLJCLin: return direct_go<TriLjcVjp<true>, 2, 2>(a, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace nbody

@@ -38,23 +38,114 @@ struct VjpFinalizeArgs {
   // arrays of stride `stride`, see VjpArgs) and the word holding 2^-S; null: slots
   const long long *acc64;
   const double *fx_inv;
+  TriGeom tri;        // streamed triangle kernels' slots (as in FinalizeArgs), or h = 0
+  int lam_is_u;       // LJC: lam holds u = lam / m already
+  // Per-type sums: each block adds its own to its row of type_part over the VJPs of one
+  // call (kTypeFirst: starts the row); in the last one (kTypeLast) the block that finishes
+  // last adds the rows to the caller's. One reduction over the blocks per call: it is a
+  // chain of fence, atomic and dependent loads, 4 us of a reverse step's 88 at 8192 atoms.
+  int type_ends;
+  unsigned *ticket;
+  double *grad_types;
+  int ntypes;
 };
+enum : int { kTypeFirst = 1, kTypeLast = 2 };
 
-__global__ void __launch_bounds__(256) vjp_finalize_kernel(const VjpFinalizeArgs f) {
+// Sums of a particle's streamed-kernel slots, by SPLIT threads each adding one of SPLIT
+// equal runs of them (SPLIT x 64 threads, particles first); the first then holds the
+// total and returns true. The second row of each slot lies `bstride` further (TWO).
+constexpr int kSlotParts = 64;  // particles per block
+template <int SPLIT>
+__device__ __forceinline__ bool tri_slot_sums(const float4 *part, long long stride,
+                                              long long bstride, const TriGeom &g, bool two,
+                                              int i, int run, float4 &hA, float4 &oA, float4 &hB,
+                                              float4 &oB) {
+  __shared__ float4 runs[4][SPLIT - 1][kSlotParts];
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  hA = oA = hB = oB = zero;
+  const int row = min(i, g.n - 1) / (64 * g.h);
+  int first, shares;
+  tri_row_shares(g, row, first, shares);
+  const int below = row + 1, count = below + shares;
+  const int k0 = count * run / SPLIT, k1 = count * (run + 1) / SPLIT;
+  auto add = [](float4 &h, float4 &o, const float4 &a) {
+    comp_add(h.x, o.x, a.x);
+    comp_add(h.y, o.y, a.y);
+    comp_add(h.z, o.z, a.z);
+    comp_add(h.w, o.w, a.w);
+  };
+  auto at = [&](int c) {  // source-side slots 0 .. row, then the target-side ones from nb on
+    return (long long)(c < below ? c : g.nb + c - below) * stride + i;
+  };
+  constexpr int U = 8;  // slots on their way
+  if (i < g.n) {
+    for (int c = k0; c < k1; c += U) {
+      float4 a[U], b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        a[u] = c + u < k1 ? part[at(c + u)] : zero;
+        b[u] = two && c + u < k1 ? part[at(c + u) + bstride] : zero;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        add(hA, oA, a[u]);
+        if (two) add(hB, oB, b[u]);
+      }
+    }
+  }
+  const int p = threadIdx.x - run * kSlotParts;
+  if (run > 0) {
+    runs[0][run - 1][p] = hA;
+    runs[1][run - 1][p] = oA;
+    runs[2][run - 1][p] = hB;
+    runs[3][run - 1][p] = oB;
+  }
+  __syncthreads();
+  if (run > 0) return false;
+  auto plus = [](float4 &o, const float4 &l) {
+    o.x += l.x;
+    o.y += l.y;
+    o.z += l.z;
+    o.w += l.w;
+  };
+#pragma unroll
+  for (int q = 0; q < SPLIT - 1; ++q) {
+    add(hA, oA, runs[0][q][p]);
+    plus(oA, runs[1][q][p]);
+    add(hB, oB, runs[2][q][p]);
+    plus(oB, runs[3][q][p]);
+  }
+  return true;
+}
+
+// SPLIT 1: the partials of the tile and direct kernels, 256 particles per block; SPLIT 4:
+// those of the streamed triangle kernels, 64 particles per block.
+template <int SPLIT>
+__global__ void __launch_bounds__(256) vjp_finalize_kernel(
+    const __grid_constant__ VjpFinalizeArgs f) {
+  if (SPLIT > 1) griddep_launch();
   griddep_start();
-  const int i = blockIdx.x * 256 + threadIdx.x;
-  double tv[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (i < f.n) {
+  constexpr int kParts = 256 / SPLIT;
+  const int run_of = SPLIT > 1 ? threadIdx.x / kParts : 0;
+  const int i = blockIdx.x * kParts + threadIdx.x - run_of * kParts;
+  int my_type = -1;  // this particle's type, and its terms of the type's gradients
+  double my_sigma = 0.0, my_eps = 0.0;
+  float4 hA, oA, hB, oB;
+  bool mine = true;
+  if constexpr (SPLIT > 1)
+    mine = tri_slot_sums<SPLIT>(f.part_hi, f.stride, f.bstride, f.tri,
+                                f.law != NBODY_LAW_GRAV, i, run_of, hA, oA, hB, oB);
+  if (mine && i < f.n) {
     // part_lo == nullptr: partials without low parts (Newton-symmetric gravity tiles)
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 hA = zero, oA = zero, hB = zero, oB = zero;
+    if (SPLIT == 1) hA = oA = hB = oB = zero;
     const bool lj = (f.law == NBODY_LAW_LJC || f.law == NBODY_LAW_LJC_LINEAR);
     const int sp = f.sym_split > 1 ? f.sym_split : 1;
     const int own_b = sp > 1 ? i / f.sym_block : 0;
     const int own_s = sp > 1 ? ((i - own_b * f.sym_block) >> 1) / (f.sym_block / 2 / sp) : 0;
     const int below = own_b;        // slots own_s, own_s + sp, ... below the own block
     const int k_all = own_b * sp;   // every slot from here on
-    const int count = f.acc64 ? 0 : below + (f.slices - k_all);
+    const int count = f.acc64 || SPLIT > 1 ? 0 : below + (f.slices - k_all);
     auto offset = [&](int c) {
       const int k = c < below ? c * sp + own_s : k_all + (c - below);
       return (long long)k * f.stride + i;
@@ -117,7 +208,11 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(const VjpFinalizeArgs
       gm = -f.G * aw;
     } else {
       const float4 x = f.pos[i];
-      const float4 u = f.lam[i];
+      float4 u = f.lam[i];
+      if (!f.lam_is_u) {
+        const float inv = 1.0f / x.w;
+        u = make_float4(u.x * inv, u.y * inv, u.z * inv, 0.0f);
+      }
       const float bx = hB.x + oB.x, by = hB.y + oB.y, bz = hB.z + oB.z, bw = hB.w + oB.w;
       gx = ax;
       gy = ay;
@@ -126,9 +221,14 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(const VjpFinalizeArgs
       const float4 q = f.prm[i];
       const int t = int(q.w);
       if (f.type_part && t >= 0 && t < 4) {
-        const double e2 = double(q.z) * double(q.z);  // 24 eps_k
-        tv[t] = -3.0 * double(aw) * f.alpha;
-        tv[4 + t] = -12.0 / e2 * double(bw) * f.alpha;
+        // 1 / e2, e2 = (24 eps_k): the FP32 reciprocal and two Newton steps
+        const double e2 = double(q.z) * double(q.z);
+        double r = double(1.0f / float(e2));
+        r = r * (2.0 - e2 * r);
+        r = r * (2.0 - e2 * r);
+        my_type = t;
+        my_sigma = double(aw);
+        my_eps = double(bw) * r;
       }
     }
     float4 gxo = f.accumulate ? f.grad_x[i] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -150,85 +250,164 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(const VjpFinalizeArgs
     }
   }
   if (f.type_part) {
-    // fixed-order block sum of the 8 per-type fields
-    __shared__ double red[8][8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-#pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) tv[k] += __shfl_down_sync(0xffffffffu, tv[k], off);
-      if (lane == 0) red[warp][k] = tv[k];
+    // Sums over the block's particles, then over the blocks, one field per warp, in a
+    // fixed order (FP64 runs at two lanes a cycle per SM: the adds are few on purpose).
+    __shared__ double val[2][kParts];
+    __shared__ int type[kParts];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, field = threadIdx.x >> 5;
+    const int which = field >> 2, t = field & 3;  // which: 0 sigma, 1 epsilon
+    if (mine) {
+      const int p = threadIdx.x - run_of * kParts;
+      type[p] = my_type;
+      val[0][p] = my_sigma;
+      val[1][p] = my_eps;
     }
     __syncthreads();
-    if (threadIdx.x < 8) {
-      double s = 0.0;
-      for (int w = 0; w < 8; ++w) s += red[w][threadIdx.x];
-      f.type_part[(size_t)blockIdx.x * 8 + threadIdx.x] = s;
+    auto warp_sum = [](double s) {
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+      return s;
+    };
+    double s = 0.0;
+#pragma unroll
+    for (int p = 0; p < kParts; p += 32)
+      if (type[p + lane] == t) s += val[which][p + lane];
+    s = warp_sum(s);
+    if (lane == 0) {
+      double *row = f.type_part + (size_t)blockIdx.x * 8 + field;
+      s *= (which ? -12.0 : -3.0) * f.alpha;
+      *row = f.type_ends & kTypeFirst ? s : *row + s;
     }
+    if (!(f.type_ends & kTypeLast)) return;
+    // the block that finishes last adds the blocks' rows
+    __threadfence();  // this block's row is visible before its ticket is taken
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(f.ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const volatile double *rows = f.type_part;
+    s = 0.0;
+    for (int b = lane; b < int(gridDim.x); b += 32) s += rows[(size_t)b * 8 + field];
+    s = warp_sum(s);
+    if (lane == 0 && t < f.ntypes) f.grad_types[which * f.ntypes + t] += s;
   }
 }
 
-// GAJ: fixed-order compensated sum of the per-slice partials of A (acceleration)
-// and B (jerk), scaled by G.
-// acc64 (with inv = 2^-S): the exact fixed-point sums of the Newton-symmetric
-// tiles, sixteen int64 arrays of stride `stride` (acceleration x, y, z, -, their
-// fractions, then the same four and four for the jerk), rounded once; else null.
-__global__ void __launch_bounds__(256) gaj_finalize_kernel(const float4 *part_hi,
-                                                           const float4 *part_lo,
-                                                           long long stride, long long bstride,
-                                                           int slices, int n, float G,
-                                                           float4 *acc, float4 *jerk,
-                                                           const long long *acc64,
-                                                           const double *inv) {
-  const int i = blockIdx.x * 256 + threadIdx.x;
-  if (i >= n) return;
-  if (acc64) {
-    const double iv = *inv;
-    auto v = [&](int c) {
-      return G * float(fixed_value(acc64[c * stride + i], acc64[(4 + c) * stride + i], iv));
-    };
-    auto w = [&](int c) {
-      return G * float(fixed_value(acc64[(8 + c) * stride + i], acc64[(12 + c) * stride + i],
-                                   iv));
-    };
-    acc[i] = make_float4(v(0), v(1), v(2), 0.0f);
-    jerk[i] = make_float4(w(0), w(1), w(2), 0.0f);
-    return;
-  }
-  // part_lo == nullptr: partials without low parts (Newton-symmetric tiles)
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 hA = part_hi[i], oA = part_lo ? part_lo[i] : zero;
-  float4 hB = part_hi[bstride + i], oB = part_lo ? part_lo[bstride + i] : zero;
-  for (int k = 1; k < slices; ++k) {
-    const long long o = (long long)k * stride + i;
-    const float4 a = part_hi[o], la = part_lo ? part_lo[o] : zero, b = part_hi[bstride + o],
-                 lb = part_lo ? part_lo[bstride + o] : zero;
-    comp_add(hA.x, oA.x, a.x);
-    comp_add(hA.y, oA.y, a.y);
-    comp_add(hA.z, oA.z, a.z);
-    comp_add(hB.x, oB.x, b.x);
-    comp_add(hB.y, oB.y, b.y);
-    comp_add(hB.z, oB.z, b.z);
-    oA.x += la.x;
-    oA.y += la.y;
-    oA.z += la.z;
-    oB.x += lb.x;
-    oB.y += lb.y;
-    oB.z += lb.z;
-  }
-  acc[i] = make_float4(G * (hA.x + oA.x), G * (hA.y + oA.y), G * (hA.z + oA.z), 0.0f);
-  jerk[i] = make_float4(G * (hB.x + oB.x), G * (hB.y + oB.y), G * (hB.z + oB.z), 0.0f);
+// Acceleration + jerk: the partials of A (acceleration) and B (jerk) added in a fixed
+// order, compensated, and scaled by G; in a Hermite step also the corrector and, unless
+// it is the last step, the next one's predictor (one launch for the three).
+struct GajFinalizeArgs {
+  const float4 *part_hi;
+  const float4 *part_lo;  // null: partials without low parts
+  long long stride;
+  long long bstride;
+  int slices;
+  int n;
+  float G;
+  float4 *acc;   // in: acceleration and jerk at the step's start (corrector); out
+  float4 *jerk;
+  // the exact fixed-point sums of the Newton-symmetric tiles (with inv = 2^-S): sixteen
+  // int64 arrays of stride `stride` (acceleration x, y, z, -, their fractions, then the
+  // same four and four for the jerk), rounded once; else null
+  const long long *acc64;
+  const double *inv;
+  TriGeom tri;   // streamed triangle kernels' slots, or h = 0
+  float4 *pos;   // corrector: the step's start, and its end; null: none
+  float4 *vel;
+  float dt;
+  float4 *xp;    // the next step's predicted positions and velocities, or null
+  float4 *vp;
+};
+
+// Hermite predictor: x_p = x + dt (v + dt (a/2 + dt j/6)), v_p = v + dt (a + dt j/2).
+__device__ __forceinline__ void hermite_predict(const float4 &x, const float4 &v,
+                                                const float4 &a, const float4 &j, float dt,
+                                                float4 &xp, float4 &vp) {
+  const float h2 = 0.5f * dt, h6 = dt * (1.0f / 6.0f);
+  xp = make_float4(fmaf(dt, fmaf(dt, fmaf(h6, j.x, 0.5f * a.x), v.x), x.x),
+                   fmaf(dt, fmaf(dt, fmaf(h6, j.y, 0.5f * a.y), v.y), x.y),
+                   fmaf(dt, fmaf(dt, fmaf(h6, j.z, 0.5f * a.z), v.z), x.z), x.w);
+  vp = make_float4(fmaf(dt, fmaf(h2, j.x, a.x), v.x), fmaf(dt, fmaf(h2, j.y, a.y), v.y),
+                   fmaf(dt, fmaf(h2, j.z, a.z), v.z), 0.0f);
 }
 
-// Sum per-block type partials in order and add them into out[0..2*ntypes).
-__global__ void type_reduce_kernel(const double *part, int nblk, int ntypes, double *out) {
+// SPLIT as in vjp_finalize_kernel.
+template <int SPLIT>
+__global__ void __launch_bounds__(256) gaj_finalize_kernel(
+    const __grid_constant__ GajFinalizeArgs f) {
+  if (SPLIT > 1) griddep_launch();
   griddep_start();
-  const int k = threadIdx.x;
-  if (k >= 8) return;
-  double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += part[(size_t)b * 8 + k];
-  const int t = k & 3, which = k >> 2;  // 0: sigma, 1: eps
-  if (t < ntypes) out[which * ntypes + t] += s;
+  constexpr int kParts = 256 / SPLIT;
+  const int run_of = SPLIT > 1 ? threadIdx.x / kParts : 0;
+  const int i = blockIdx.x * kParts + threadIdx.x - run_of * kParts;
+  float4 hA, oA, hB, oB;
+  if constexpr (SPLIT > 1) {
+    if (!tri_slot_sums<SPLIT>(f.part_hi, f.stride, f.bstride, f.tri, true, i, run_of, hA, oA, hB,
+                              oB))
+      return;
+  }
+  if (i >= f.n) return;
+  float4 a1, j1;
+  if (SPLIT == 1 && f.acc64) {
+    const double iv = *f.inv;
+    auto v = [&](int c) {
+      return f.G * float(fixed_value(f.acc64[c * f.stride + i], f.acc64[(4 + c) * f.stride + i],
+                                     iv));
+    };
+    a1 = make_float4(v(0), v(1), v(2), 0.0f);
+    j1 = make_float4(v(8), v(9), v(10), 0.0f);
+  } else {
+    if (SPLIT == 1) {
+      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+      hA = f.part_hi[i];
+      oA = f.part_lo ? f.part_lo[i] : zero;
+      hB = f.part_hi[f.bstride + i];
+      oB = f.part_lo ? f.part_lo[f.bstride + i] : zero;
+      for (int k = 1; k < f.slices; ++k) {
+        const long long o = (long long)k * f.stride + i;
+        const float4 a = f.part_hi[o], la = f.part_lo ? f.part_lo[o] : zero;
+        const float4 b = f.part_hi[f.bstride + o];
+        const float4 lb = f.part_lo ? f.part_lo[f.bstride + o] : zero;
+        comp_add(hA.x, oA.x, a.x);
+        comp_add(hA.y, oA.y, a.y);
+        comp_add(hA.z, oA.z, a.z);
+        comp_add(hB.x, oB.x, b.x);
+        comp_add(hB.y, oB.y, b.y);
+        comp_add(hB.z, oB.z, b.z);
+        oA.x += la.x;
+        oA.y += la.y;
+        oA.z += la.z;
+        oB.x += lb.x;
+        oB.y += lb.y;
+        oB.z += lb.z;
+      }
+    }
+    a1 = make_float4(f.G * (hA.x + oA.x), f.G * (hA.y + oA.y), f.G * (hA.z + oA.z), 0.0f);
+    j1 = make_float4(f.G * (hB.x + oB.x), f.G * (hB.y + oB.y), f.G * (hB.z + oB.z), 0.0f);
+  }
+  if (f.pos) {
+    // Hermite corrector (time-symmetric form):
+    //   v1 = v + dt/2 (a + a1) + dt^2/12 (j - j1),
+    //   x1 = x + dt/2 (v + v1) + dt^2/12 (a - a1)
+    const float4 x = f.pos[i], v = f.vel[i], a = f.acc[i], j = f.jerk[i];
+    const float h = 0.5f * f.dt, q = f.dt * f.dt * (1.0f / 12.0f);
+    float4 v1, x1;
+    v1.x = fmaf(q, j.x - j1.x, fmaf(h, a.x + a1.x, v.x));
+    v1.y = fmaf(q, j.y - j1.y, fmaf(h, a.y + a1.y, v.y));
+    v1.z = fmaf(q, j.z - j1.z, fmaf(h, a.z + a1.z, v.z));
+    v1.w = v.w;
+    x1.x = fmaf(q, a.x - a1.x, fmaf(h, v.x + v1.x, x.x));
+    x1.y = fmaf(q, a.y - a1.y, fmaf(h, v.y + v1.y, x.y));
+    x1.z = fmaf(q, a.z - a1.z, fmaf(h, v.z + v1.z, x.z));
+    x1.w = x.w;
+    f.pos[i] = x1;
+    f.vel[i] = v1;
+    if (f.xp) hermite_predict(x1, v1, a1, j1, f.dt, f.xp[i], f.vp[i]);
+  }
+  f.acc[i] = a1;
+  f.jerk[i] = j1;
 }
 
 // Fixed-point accumulation of the symmetric gravity VJP: the accumulators that

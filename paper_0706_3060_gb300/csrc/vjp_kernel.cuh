@@ -49,12 +49,6 @@ struct VjpArgs {
   const float *fscale;
 };
 
-__device__ __forceinline__ float rcp_hw(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
 template <bool MASK>
 __device__ __forceinline__ void grav_vjp_pair(const float4 pj, const float4 lj, float xk,
                                               float yk, float zk, float mk, float lkx, float lky,
