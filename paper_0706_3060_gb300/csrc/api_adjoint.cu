@@ -121,6 +121,7 @@ int launch_untiled(const float4 *pos, const float4 *prm, const float4 *vec, int 
     t.p1 = prm;
     t.p2 = vec;
     t.part = sc.part_hi;
+    t.stride = n;
     t.ostride = sc.bstride;
     t.eps2 = p.eps2;
     t.geom = sc.geom;

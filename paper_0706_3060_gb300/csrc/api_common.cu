@@ -702,6 +702,7 @@ int launch_forces(const float4 *pos, const float4 *prm, int law, uint32_t flags,
     t.p0 = pos;
     t.p1 = prm;
     t.part = part_hi;
+    t.stride = n;
     t.eps2 = eps2;
     t.geom = p.geom;
     t.pdl = chained ? 1 : 0;

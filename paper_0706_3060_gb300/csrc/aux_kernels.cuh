@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kFinThreads * SPLIT) finalize_kernel(
     const int row = min(i, f.n - 1) / (64 * f.tri.h);
     int first, shares;
     tri_row_shares(f.tri, row, first, shares);
-    below = row + 1;
+    below = row;
     k0 = (below + shares) * run_of / SPLIT;
     k1 = (below + shares) * (run_of + 1) / SPLIT;
   }
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kFinThreads * SPLIT) finalize_kernel(
   if constexpr (SPLIT > 1) {
     __shared__ float4 runs[2][SPLIT - 1][kFinThreads];
     if (i < f.n) {
-      // the source-side slots 0 .. row, then the target-side slots from nb on
+      // the source-side slots 0 .. row - 1, then the target-side slots from nb on
       run(k0, min(k1, below) - k0, 1);
       run(f.tri.nb + max(k0, below) - below, k1 - max(k0, below), 1);
     }

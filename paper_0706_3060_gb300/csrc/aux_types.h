@@ -66,7 +66,7 @@ struct FinalizeArgs {
   int jn_words;
   int rezero;  // atomic plans: zero the accumulators after reading them
   // Streamed triangle kernels (tri_plan.h): particle i of row b counts the slots
-  // 0 .. b (source side) and nb .. nb + (shares of row b) - 1 (target side).
+  // 0 .. b - 1 (source side) and nb .. nb + (shares of row b) - 1 (target side).
   // tri.h == 0: another kernel's slots.
   TriGeom tri;
   // With kFinDiag: also add the block rows of diag_part into diag_out (8 doubles)

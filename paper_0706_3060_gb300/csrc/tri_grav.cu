@@ -7,11 +7,12 @@ namespace nbody {
 const TriDesc *tri_grav(int64_t n) {
   // Rows of 384 targets leave a small system more units for equal shares; rows of 512
   // spend fewer instructions per pair on moving the sources. Kernel times (us), 384 /
-  // 512: 28.7 / 30.7 at 8192, 82.0 / 84.0 at 16384, 678 / 670 at 50021, 2162 / 2128 at
-  // 90000 (rows of 256, four CTAs per SM: 28.7, 85.0, 713, 2274).
+  // 512: 13.3 / 13.6 at 5000, 24.0 / 24.6 at 8192, 46.1 / 45.5 at 12288, 77.5 / 76.6 at
+  // 16384, 294 / 287 at 32768, 2170 / 2116 at 90000 (rows of 256: 15.7, 24.1, 48.5, 82.4,
+  // 314, 2328).
   static const TriDesc small = TriImpl<TriGrav, 6, 2, true>::desc();
   static const TriDesc large = TriImpl<TriGrav, 8, 2, true>::desc();
-  return n < 32768 ? &small : &large;
+  return n < 12288 ? &small : &large;
 }
 
 }  // namespace nbody

@@ -21,17 +21,18 @@
 // 2 H targets per step share them. Pairs of targets instead of pairs of sources in the
 // f32x2 halves halve the registers per target (no duplicated target words), so a lane
 // holds up to 16 targets at 8 warps per SM. Equal shares leave no partial wave: all CTAs
-// are resident from the start and end within 10% of each other. Two CTAs of four warps
+// are resident from the start (taken from a queue in smaller pieces instead, 3 to 6%
+// more: 82 us against 77.5 at 16384, 298 against 287 at 32768). Two CTAs of four warps
 // per SM: one of eight, whose warps keep step with each other, took 5% longer.
-// Leapfrog steps inside a call (us), block-pair tile -> here: gravity 36.4 -> 29.3 at
-// 8192, 91.8 -> 83.3 at 16384, 308 -> 306 at 32768; LJC 44.9 -> 39.2, 129.6 -> 119.2,
-// 475 -> 445, and 1831 -> 1738 at 65536 (80% of the FP32 lane peak).
+// Leapfrog steps inside a call (us), block-pair tile -> here: gravity 36.4 -> 28.2 at
+// 8192, 91.8 -> 81.9 at 16384, 308 -> 295 at 32768; LJC 44.9 -> 37.1, 129.6 -> 117.3,
+// 475 -> 444, and 1831 -> 1738 at 65536 (80% of the FP32 lane peak).
 //
 // Sums. A target's sum is plain FP32 over at most 128 sources, then over at most four
 // such sums of a window of 64 groups, then over the four warps, each in order, and over
 // the windows of a share with TwoSum. A source's sum is plain FP32 over the 2 H targets
 // of a step and then over the steps. Partials go, per row b,
-//   * source side: one per row and particle, to slot b;
+//   * source side: one per row and particle beyond it, to slot b;
 //   * target side: one per share and target, to slot nb + (share - first share of
 //     the row);
 // each written once, so the finalize adds a particle's slots in a fixed order
@@ -55,7 +56,8 @@ struct TriArgs {
   const float4 *p0;  // (x, y, z, m)
   const float4 *p1;  // LJC parameters
   const float4 *p2;  // velocities, lambda, u (VJP and jerk laws)
-  float4 *part;      // [slot][n], kSums floats each: one float4, or two (hi at ostride)
+  float4 *part;      // [slot][stride], kSums floats each: one float4, or two (hi at ostride)
+  long long stride;
   long long ostride; // elements from the first float4 of a partial to its second
   float eps2;
   TriGeom geom;
@@ -83,7 +85,7 @@ __device__ __forceinline__ int tri_place(int t) {
 template <class L>
 __device__ __forceinline__ void tri_store(const TriArgs &a, int slot, int i,
                                           const float (&v)[L::kSums]) {
-  const long long o = (long long)slot * a.geom.n + i;
+  const long long o = (long long)slot * a.stride + i;
   if constexpr (L::kSums % 3 == 0) {
     a.part[o] = make_float4(v[0], v[1], v[2], 0.0f);
     if constexpr (L::kSums == 6) a.part[o + a.ostride] = make_float4(v[3], v[4], v[5], 0.0f);
@@ -93,13 +95,12 @@ __device__ __forceinline__ void tri_store(const TriArgs &a, int slot, int i,
   }
 }
 
-// STEPS steps of one source group from step s0 on, against the row's targets in
-// registers; the lane starts with source (lane + s0) & 31 of the group in S. On return
-// B holds the source-side sums of source (lane + s0 + STEPS) & 31 over these steps,
-// before their sign change. DIAG: the group is the row's own-th.
-template <class L, int H, bool DIAG, int STEPS>
-__device__ __forceinline__ void tri_group(float eps2, int own, int s0,
-                                          const float2 (&T)[H][L::kWords],
+// STEPS steps of one source group beyond the row, from step s0 on, against the row's
+// targets in registers; the lane starts with source (lane + s0) & 31 of the group in S. On
+// return B holds the source-side sums of source (lane + s0 + STEPS) & 31 over these steps,
+// before their sign change.
+template <class L, int H, int STEPS>
+__device__ __forceinline__ void tri_group(float eps2, const float2 (&T)[H][L::kWords],
                                           float2 (&A)[H][L::kSums], float (&B)[L::kSums],
                                           float (&S)[L::kWords]) {
   const int next = (threadIdx.x & 31) + 1;
@@ -111,32 +112,39 @@ __device__ __forceinline__ void tri_group(float eps2, int own, int s0,
     float J[2 * L::kSums];  // over this step's targets: even ones J[2c], odd ones J[2c+1]
 #pragma unroll
     for (int c = 0; c < 2 * L::kSums; ++c) J[c] = 0.0f;
-    if constexpr (!DIAG) {
 #pragma unroll
-      for (int r = 0; r < H; ++r) L::template pair<false>(S, T[r], A[r], J, e2);
-    } else {
-      // register groups below the source's own hold pairs not yet counted; with its
-      // own it is summed one-sided (source and target meet twice there; the self
-      // pair, met in step 0, is dropped); those above wait for their source groups
-      // (skipped two at a time)
-      const int mine = own >> 1;
-#pragma unroll
-      for (int r0 = 0; r0 < H; r0 += 2) {
-        if (r0 <= mine) {
-#pragma unroll
-          for (int r = r0; r < (r0 + 2 < H ? r0 + 2 : H); ++r) {
-            const bool self = r == mine && st + s0 == 0;
-            L::template pair<true>(S, T[r], A[r], J, e2, r <= mine && !(self && !(own & 1)),
-                                   r <= mine && !(self && (own & 1)), r < mine);
-          }
-        }
-      }
-    }
+    for (int r = 0; r < H; ++r) L::template pair<false>(S, T[r], A[r], J, e2);
 #pragma unroll
     for (int c = 0; c < L::kSums; ++c)
       B[c] = __shfl_sync(0xffffffffu, B[c] + (J[2 * c] + J[2 * c + 1]), next);
 #pragma unroll
     for (int c = 0; c < L::kWords; ++c) S[c] = __shfl_sync(0xffffffffu, S[c], next);
+  }
+}
+
+// The same for the row's own-th own group, one-sided: the row's pairs are met in both
+// orders, each time for the target alone, and only a lane's first step can meet itself.
+// Twice the pairs, but no source side, and one straight loop: masking what was counted
+// already (each own pair once, register groups skipped two at a time) took 2.5 us a unit
+// against 1.7 of a unit beyond the row (gravity), waiting on the few pairs in flight.
+template <class L, int H, int STEPS>
+__device__ __forceinline__ void tri_own_group(float eps2, int own, int s0,
+                                              const float2 (&T)[H][L::kWords],
+                                              float2 (&A)[H][L::kSums], float (&S)[L::kWords]) {
+  const int next = (threadIdx.x & 31) + 1;
+  const float2 e2 = bcast(eps2);
+  float J[2 * L::kSums];  // not used
+  const int self = s0 == 0 ? own >> 1 : -1;
+#pragma unroll
+  for (int r = 0; r < H; ++r)
+    L::template pair<true, false>(S, T[r], A[r], J, e2, !(r == self && !(own & 1)),
+                                  !(r == self && (own & 1)));
+#pragma unroll 1
+  for (int st = 1; st < STEPS; ++st) {
+#pragma unroll
+    for (int c = 0; c < L::kWords; ++c) S[c] = __shfl_sync(0xffffffffu, S[c], next);
+#pragma unroll
+    for (int r = 0; r < H; ++r) L::template pair<false, false>(S, T[r], A[r], J, e2);
   }
 }
 
@@ -248,14 +256,22 @@ __device__ __forceinline__ void tri_run(const TriArgs &a, int row, int d0, int d
         } else {
           L::load(a.p0, a.p1, a.p2, i, n, S);
         }
-        tri_group<L, H, DIAG, 32>(a.eps2, gg - 2 * H * row, 0, T, A, v, S);
-        source_sums();
-        if (i < n) tri_store<L>(a, row, i, v);
+        if constexpr (DIAG) {
+          tri_own_group<L, H, 32>(a.eps2, gg - 2 * H * row, 0, T, A, S);
+        } else {
+          tri_group<L, H, 32>(a.eps2, T, A, v, S);
+          source_sums();
+          if (i < n) tri_store<L>(a, row, i, v);
+        }
       }
       for (int m = 0; m < left; ++m) {  // its eight steps of each left-over group
         const int gg = g + 4 * quads + m, s0 = 8 * warp;
         L::load(a.p0, a.p1, a.p2, gg * kTriGroup + ((lane + s0) & 31), n, S);
-        tri_group<L, H, DIAG, 8>(a.eps2, gg - 2 * H * row, s0, T, A, v, S);
+        if constexpr (DIAG) {
+          tri_own_group<L, H, 8>(a.eps2, gg - 2 * H * row, s0, T, A, S);
+          continue;
+        }
+        tri_group<L, H, 8>(a.eps2, T, A, v, S);
         source_sums();
 #pragma unroll
         for (int c = 0; c < NS; ++c)

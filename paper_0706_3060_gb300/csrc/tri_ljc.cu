@@ -10,8 +10,9 @@ using Law = TriLjc<false, POT, PRECISE>;
 }
 
 const TriDesc *tri_ljc(int64_t n) {
-  // As for gravity. Kernel times (us, constant dielectric), rows of 256 / 384: 36.9 /
-  // 38.9 at 8192, 122.8 / 118.8 at 16384, 1043 / 1003 at 50021, 3343 / 3208 at 90000.
+  // As for gravity. Kernel times (us), rows of 256 / 384: 16.2 / 17.6 at 5000, 32.6 / 33.6
+  // at 8192, 68.4 / 65.6 at 12288, 116.0 / 112.5 at 16384, 449 / 432 at 32768, 3342 / 3200
+  // at 90000.
   static const TriDesc small = TriImpl<Law, 4, 2, true>::desc();
   static const TriDesc large = TriImpl<Law, 6, 2, true>::desc();
   return n < 12288 ? &small : &large;

@@ -1,16 +1,16 @@
 // tri_vjp.cu -- streamed triangle and direct kernels of acceleration + jerk (Table 1
 // "Gravity (accel & jerk)") and of the gravity and LJC force VJPs.
 //
-// What bounds them: the packed FP32 unit (33, 35 and 64 operations per pair; 0.71, 0.72
-// and 0.78 of its rate at 32768), of which the three-operand multiply-adds take a sixth
-// more than the others. Rows of 256 targets: 226, 196 and 255 registers at two CTAs per
+// What bounds them: the packed FP32 unit (33, 35 and 64 operations per pair; 0.72, 0.74
+// and 0.81 of its rate at 32768), of which the three-operand multiply-adds take a sixth
+// more than the others. Rows of 256 targets: 231, 196 and 255 registers at two CTAs per
 // SM; rows of 384 spill (jerk: 642 us at 32768 against 614) or gain nothing (gravity VJP:
-// 637 against 642 at 32768, 165 against 166 at 16384, 48.0 against 46.4 at 8192), rows of
-// 128 move the sources twice as often (LJC VJP: 1153 us at 32768 against 1065).
+// 47.2 us against 44.3 at 8192, 163 against 162 at 16384, 635 against 629 at 32768), rows
+// of 128 move the sources twice as often (LJC VJP: 1153 us at 32768 against 1065).
 // Per step with the finalize, against the block-pair tiles (us):
-//   Hermite 8192 49.2 / 79.2, 16384 165 / 215, 32768 630 / 685
-//   gravity reverse step 4096 21.4 / 27.4, 8192 50.1 / 61.7, 16384 170 / 185
-//   LJC reverse step 4096 34.8 / 46.3, 8192 82 / 105, 32768 1097 / 2186
+//   Hermite 8192 46.6 / 79.2, 16384 163 / 215, 32768 629 / 685
+//   gravity reverse step 4096 20.8 / 27.4, 8192 47.9 / 61.7, 16384 167 / 185
+//   LJC reverse step 4096 33.1 / 46.3, 8192 78.4 / 105, 32768 1082 / 2186
 #include "api_common.h"
 #include "direct_impl.h"
 #include "tri_impl.h"

@@ -66,7 +66,7 @@ __device__ __forceinline__ bool tri_slot_sums(const float4 *part, long long stri
   const int row = min(i, g.n - 1) / (64 * g.h);
   int first, shares;
   tri_row_shares(g, row, first, shares);
-  const int below = row + 1, count = below + shares;
+  const int below = row, count = below + shares;
   const int k0 = count * run / SPLIT, k1 = count * (run + 1) / SPLIT;
   auto add = [](float4 &h, float4 &o, const float4 &a) {
     comp_add(h.x, o.x, a.x);
@@ -74,7 +74,7 @@ __device__ __forceinline__ bool tri_slot_sums(const float4 *part, long long stri
     comp_add(h.z, o.z, a.z);
     comp_add(h.w, o.w, a.w);
   };
-  auto at = [&](int c) {  // source-side slots 0 .. row, then the target-side ones from nb on
+  auto at = [&](int c) {  // source-side slots 0 .. row - 1, then the target-side ones from nb on
     return (long long)(c < below ? c : g.nb + c - below) * stride + i;
   };
   constexpr int U = 8;  // slots on their way
