@@ -23,6 +23,11 @@ int launch_finalize(const FinalizeArgs &f, cudaStream_t s, int *nblk_out, bool p
   return NBODY_OK;
 }
 
+int launch_batch_finalize(const BatchFinalizeArgs &f, cudaStream_t s) {
+  NB_CUDA(launch_kernel(batch_finalize_kernel, (f.n + 255) / 256, 256, 0, s, true, f));
+  return NBODY_OK;
+}
+
 int launch_kick_drift(float4 *pos, float4 *vel, const float4 *acc, int n, float dt,
                       float4 *trace1, const int *sys_of, const void *sys, float4 *x_lo,
                       float4 *v_lo, cudaStream_t s) {

@@ -11,6 +11,7 @@
 
 #include "api_common.h"
 #include "aux_types.h"
+#include "tri_batch.cuh"
 
 using namespace nbody;
 
@@ -19,8 +20,12 @@ struct nbody_batch_plan {
   int sms = 0;
   std::vector<nbody_system> sys;
   int64_t total = 0;
-  const TileDesc *td = nullptr;
+  const TileDesc *td = nullptr;  // null: the streamed triangle kernel
   uint32_t flags = 0;
+  TriSeg *d_segs = nullptr;
+  int n_segs = 0;
+  int *d_row_of = nullptr;
+  RowInfo *d_rows = nullptr;
   int n_items = 0;
   int max_slices = 1;
   int grid = 0;
@@ -47,6 +52,9 @@ void free_plan(nbody_batch_plan *p) {
   if (!p) return;
   if (p->gexec) cudaGraphExecDestroy(p->gexec);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
+  cudaFree(p->d_segs);
+  cudaFree(p->d_row_of);
+  cudaFree(p->d_rows);
   cudaFree(p->d_items);
   cudaFree(p->d_sys);
   cudaFree(p->d_sys_of);
@@ -180,8 +188,10 @@ int enqueue_run(nbody_batch_plan *p, float4 *pos, float4 *vel, float4 *acc, cons
   const int total = int(p->total);
   const long long stride = p->total;
   float4 *part_hi = p->d_part;
-  // the symmetric tiles write one partial per particle and block, without low parts
-  float4 *part_lo = p->td->sym ? nullptr : p->d_part + size_t(p->max_slices) * size_t(stride);
+  // the symmetric tiles and the streamed kernel write one partial per particle and slot,
+  // without low parts
+  float4 *part_lo =
+      !p->td || p->td->sym ? nullptr : p->d_part + size_t(p->max_slices) * size_t(stride);
   const int evals = nsteps + ((flags & NBODY_ACC_VALID) && nsteps > 0 ? 0 : 1);
   // Every evaluation has its own work counter so that the graph needs no
   // reset between launches of different steps; all are zeroed up front.
@@ -191,6 +201,29 @@ int enqueue_run(nbody_batch_plan *p, float4 *pos, float4 *vel, float4 *acc, cons
   // launch (the memset before it is not a kernel).
   bool chained = false;
   auto eval = [&](int mode) -> int {
+    if (!p->td) {
+      TriBatchArgs t{};
+      t.pos = pos;
+      t.prm = prm;
+      t.part = part_hi;
+      t.stride = stride;
+      t.segs = p->d_segs;
+      t.nseg = p->n_segs;
+      t.counter = p->d_counter + counter_idx++;
+      t.grid = p->grid;
+      t.pdl = chained ? 1 : 0;
+      const TimerMark tm = timer_begin(0, s);
+      const cudaError_t e = tri_batch(t, (p->flags & NBODY_PRECISE_RSQRT) != 0, s);
+      timer_end(tm, s);
+      if (e != cudaSuccess)
+        return set_error_msg(NBODY_ECUDA, "batched force launch failed: %s",
+                             cudaGetErrorString(e));
+      chained = true;
+      return launch_batch_finalize(
+          BatchFinalizeArgs{part_hi, stride, p->d_row_of, p->d_rows, total, mode,
+                            (p->flags & NBODY_NO_COMPENSATION) ? 1 : 0, pos, vel, acc},
+          s);
+    }
     const int g = (total + 255) / 256;
     if (p->td->sym) {
       NB_CUDA(launch_kernel(interleave_systems_blocked_kernel, g, 256, 0, s, chained, pos, prm,
@@ -270,6 +303,7 @@ int nbody_batch_plan_create(const nbody_system *systems, int32_t nsys, uint32_t 
   if (tile < -1 || tile >= count) return set_error_msg(NBODY_EINVAL, "bad tile %d", tile);
   int dev = 0, sms = 0;
   NB_TRY(check_device(&dev, &sms));
+  const bool own_choice = tile < 0 && !tuned_by_caller(kTableBatched, 0);
   if (tile < 0) {
     int tj = 0;
     get_config(kTableBatched, 0, &tile, &tj);
@@ -299,22 +333,50 @@ int nbody_batch_plan_create(const nbody_system *systems, int32_t nsys, uint32_t 
       return set_error_msg(NBODY_EINVAL, "systems %d and %d overlap", order[k - 1], order[k]);
   }
 
+  // The streamed triangle kernel, where its slots fit.
+  TriBatchPlan tri;
+  if (own_choice) {
+    std::vector<TriBatchSystem> ts;
+    for (int k = 0; k < nsys; ++k)
+      ts.push_back(
+          TriBatchSystem{systems[k].offset, systems[k].n, systems[k].law, systems[k].eps2});
+    tri = tri_batch_plan(ts, sms * tri_batch_per_sm());
+    if (double(tri.slots) * double(total) * sizeof(float4) <= sym_part_cap()) td = nullptr;
+  }
+
   // Work list: one item per (system, i-tile, j-slice). Items are cut to about
   // 1/16 of the average work per persistent CTA, so that the last items leave
   // little imbalance (measured on the 512-system ensemble: kernel 595 us with
   // 1/4, 577 us with 1/8, 561 us with 1/16; the finalize grows with the slices).
-  const int occ = td->occupancy();
+  const int occ = td ? td->occupancy() : 1;
   const int grid = sms * occ;
   double work = 0.0;
   for (int k = 0; k < nsys; ++k) work += double(systems[k].n) * double(systems[k].n);
-  const double target = std::max(work / (double(grid) * 16.0), double(td->tile_i) * td->jt);
+  const double target =
+      td ? std::max(work / (double(grid) * 16.0), double(td->tile_i) * td->jt) : 1.0;
   std::vector<WorkItem> items;
   std::vector<SysInfo> info(nsys);
   std::vector<int4> sysp(nsys);
   int max_slices = 1;
   long long pairs_law[2] = {0, 0};  // pair-buffer sizes per law (packed tiles)
   long long f4_law[2] = {0, 0};     // float4 sizes of the blocked buffers (symmetric tiles)
-  for (int k = 0; k < nsys && td->sym; ++k) {
+  std::vector<int> row_of;  // streamed kernel: row of each particle, and the rows
+  std::vector<RowInfo> rows;
+  if (!td) {
+    row_of.assign(size_t(total), -1);
+    max_slices = int(tri.slots);
+  }
+  for (int k = 0; k < nsys && !td; ++k) {
+    const nbody_system &s = systems[k];
+    const int len = 64 * tri_batch_h(s.law), nb = (s.n + len - 1) / len;
+    info[k] = SysInfo{s.law, 0, s.G, s.dt};
+    for (int i = 0; i < s.n; ++i)
+      row_of[size_t(s.offset + i)] = tri.row_base[size_t(k)] + i / len;
+    for (int b = 0; b < nb; ++b)
+      rows.push_back(RowInfo{s.law, b, nb, tri.row_shares[size_t(tri.row_base[size_t(k)] + b)],
+                             s.G, s.dt});
+  }
+  for (int k = 0; k < nsys && td && td->sym; ++k) {
     // Newton-symmetric tiles: one item per block pair (bi <= bj) of each system,
     // one partial slot per block
     const nbody_system &s = systems[k];
@@ -346,7 +408,7 @@ int nbody_batch_plan_create(const nbody_system *systems, int32_t nsys, uint32_t 
         items.push_back(w);
       }
   }
-  for (int k = 0; k < nsys && !td->sym; ++k) {
+  for (int k = 0; k < nsys && td && !td->sym; ++k) {
     const nbody_system &s = systems[k];
     const int pl = (s.law == NBODY_LAW_GRAV) ? 0 : 1;  // both LJC laws share one layout
     const int pbase = int(pairs_law[pl]);
@@ -391,33 +453,35 @@ int nbody_batch_plan_create(const nbody_system *systems, int32_t nsys, uint32_t 
   p->flags = flags;
   p->n_items = int(items.size());
   p->max_slices = max_slices;
-  p->grid = std::min(grid, p->n_items);
+  p->n_segs = int(tri.segs.size());
+  p->grid = td ? std::min(grid, p->n_items) : std::min(sms * tri_batch_per_sm(), p->n_segs);
   auto fail = [&](int code) {
     free_plan(p);
     return code;
   };
   cudaError_t e = cudaSuccess;
-  if ((e = cudaMalloc(&p->d_items, sizeof(WorkItem) * items.size())) != cudaSuccess ||
-      (e = cudaMalloc(&p->d_sys, sizeof(SysInfo) * info.size())) != cudaSuccess ||
-      (e = cudaMalloc(&p->d_sys_of, sizeof(int) * sys_of.size())) != cudaSuccess ||
-      (e = cudaMalloc(&p->d_part, sizeof(float4) * (td->sym ? 1 : 2) * size_t(max_slices) *
+  // device copy of a table (an empty one: nothing)
+  auto copy = [&](auto **dst, const auto &v) {
+    const size_t bytes = sizeof(v[0]) * v.size();
+    return v.empty() || ((e = cudaMalloc(dst, bytes)) == cudaSuccess &&
+                         (e = cudaMemcpy(*dst, v.data(), bytes, cudaMemcpyHostToDevice)) ==
+                             cudaSuccess);
+  };
+  const bool packed = td && td->packed;
+  const size_t parts = !td || td->sym ? 1 : 2;  // low parts as well
+  if (!copy(&p->d_items, items) || !copy(&p->d_sys, info) || !copy(&p->d_sys_of, sys_of) ||
+      (!td && (!copy(&p->d_segs, tri.segs) || !copy(&p->d_row_of, row_of) ||
+               !copy(&p->d_rows, rows))) ||
+      (e = cudaMalloc(&p->d_part, sizeof(float4) * parts * size_t(max_slices) *
                                       size_t(total))) != cudaSuccess ||
-      (e = cudaMemcpy(p->d_items, items.data(), sizeof(WorkItem) * items.size(),
-                      cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(p->d_sys, info.data(), sizeof(SysInfo) * info.size(),
-                      cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(p->d_sys_of, sys_of.data(), sizeof(int) * sys_of.size(),
-                      cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (td->packed &&
+      (packed &&
        ((e = cudaMalloc(&p->d_jgrav, sizeof(float4) * (td->sym ? size_t(f4_law[0] + 1)
                                                                  : 2 * size_t(pairs_law[0] + 1)))) !=
             cudaSuccess ||
         (e = cudaMalloc(&p->d_jljc, sizeof(float4) * (td->sym ? size_t(f4_law[1] + 1)
                                                                 : 3 * size_t(pairs_law[1] + 1)))) !=
             cudaSuccess ||
-        (e = cudaMalloc(&p->d_sysp, sizeof(int4) * sysp.size())) != cudaSuccess ||
-        (e = cudaMemcpy(p->d_sysp, sysp.data(), sizeof(int4) * sysp.size(),
-                        cudaMemcpyHostToDevice)) != cudaSuccess))) {
+        !copy(&p->d_sysp, sysp)))) {
     cudaGetLastError();
     return fail(set_error_msg(NBODY_ENOMEM, "batch plan allocation failed: %s",
                               cudaGetErrorString(e)));

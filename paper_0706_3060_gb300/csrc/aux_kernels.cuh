@@ -309,6 +309,74 @@ __global__ void __launch_bounds__(kFinThreads * SPLIT) finalize_kernel(
   block_sum8(v, f.diag_out);
 }
 
+// Finalize of a batched run on the streamed triangle kernel: the sums of each particle's
+// slots, its acceleration, kicks and drift, as finalize_kernel. One table entry per row
+// says all that a particle needs to know (two loads before the slots; looking up the
+// system, its rows and their slots in turn, the general kernel took 33 us for 503,103
+// particles, this one 20).
+__global__ void __launch_bounds__(256) batch_finalize_kernel(
+    const __grid_constant__ BatchFinalizeArgs f) {
+  griddep_launch();
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  const int r = i < f.n ? f.row_of[i] : -1;
+  RowInfo g{};
+  if (r >= 0) g = f.rows[r];
+  griddep_start();
+  if (r < 0) return;
+  float4 x = f.pos[i], v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (f.mode & (kFinKickSync | kFinKickDrift)) v = f.vel[i];
+  float hx = 0.f, hy = 0.f, hz = 0.f, lx = 0.f, ly = 0.f, lz = 0.f;
+  const int count = g.below + g.shares;
+  constexpr int U = 4;  // slots on their way
+  for (int c = 0; c < count; c += U) {
+    float4 h[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = c + u;
+      h[u] = k < count
+                 ? f.part[(long long)(k < g.below ? k : g.nb + k - g.below) * f.stride + i]
+                 : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (f.plain) {
+        hx += h[u].x;
+        hy += h[u].y;
+        hz += h[u].z;
+      } else {
+        comp_add(hx, lx, h[u].x);
+        comp_add(hy, ly, h[u].y);
+        comp_add(hz, lz, h[u].z);
+      }
+    }
+  }
+  const float tx = hx + lx, ty = hy + ly, tz = hz + lz;
+  float4 a;
+  if (g.law == 0) {
+    a = make_float4(g.G * tx, g.G * ty, g.G * tz, -g.G * 0.0f);
+  } else {
+    const float inv_m = 1.0f / x.w;
+    a = make_float4(-tx * inv_m, -ty * inv_m, -tz * inv_m, 0.0f);
+  }
+  if (f.mode & kFinWriteAcc) f.acc[i] = a;
+  if (!(f.mode & (kFinKickSync | kFinKickDrift))) return;
+  const float h = 0.5f * g.dt;
+  auto kick = [&]() {
+    v.x = fmaf(h, a.x, v.x);
+    v.y = fmaf(h, a.y, v.y);
+    v.z = fmaf(h, a.z, v.z);
+  };
+  if (f.mode & kFinKickSync) kick();
+  if (f.mode & kFinKickDrift) {
+    kick();
+    x.x = fmaf(g.dt, v.x, x.x);
+    x.y = fmaf(g.dt, v.y, x.y);
+    x.z = fmaf(g.dt, v.z, x.z);
+    f.pos[i] = x;
+  }
+  f.vel[i] = v;
+}
+
 // Scale of the fixed-point mode (fixed_scale_of) for the one-sided fixed-point
 // tiles: one block; the mass sum runs in FP64 in a fixed order.
 __global__ void __launch_bounds__(256) fixed_scale_kernel(const float4 *pos, int n, float eps2,

@@ -15,11 +15,36 @@ struct SysInfo {
   float dt;
 };
 
+// Per-row data of a batched run on the streamed triangle kernel: a particle of the row
+// counts the slots 0 .. below - 1 and nb .. nb + shares - 1.
+struct RowInfo {
+  int law;
+  int below;
+  int nb;
+  int shares;
+  float G;
+  float dt;
+};
+
 enum : int {
   kFinWriteAcc = 1,   // store acc (and acc_lo)
   kFinKickSync = 2,   // v += dt/2 a       (completes the previous step)
   kFinDiag = 4,       // FP64 diagnostics with the synchronized velocity
   kFinKickDrift = 8,  // v += dt/2 a; x += dt v   (starts the next step)
+};
+
+// A batched run's finalize (batch_finalize_kernel).
+struct BatchFinalizeArgs {
+  const float4 *part;
+  long long stride;
+  const int *row_of;  // row of each particle (-1: in no system)
+  const RowInfo *rows;
+  int n;
+  int mode;
+  int plain;
+  float4 *pos;
+  float4 *vel;
+  float4 *acc;
 };
 
 struct FinalizeArgs {
