@@ -22,11 +22,14 @@ COULOMB_K = 332.0637  # kcal A / (mol e^2): units A, kcal/mol, e, amu (AKMA time
 
 
 _tuned_done = False
+_loaded = None
 
 
 def _lib():
     """The loaded library, with the stored tuning table of this GPU installed once."""
-    global _tuned_done
+    global _tuned_done, _loaded
+    if _loaded is not None:
+        return _loaded
     lib = load()
     if not _tuned_done:
         _tuned_done = True
@@ -35,25 +38,36 @@ def _lib():
             tune.load_cache()
         except Exception:  # a missing or foreign cache only means default tiles
             pass
+    _loaded = lib
     return lib
 
 
+# A force call on a thousand particles takes the GPU 3 us; what Python does around it is
+# kept short: addresses and streams go to ctypes as plain integers, and the current
+# stream is read as its handle, not through a Stream object (2.3 us -> 0.3). A call of
+# forces() at 1024: 13.4 us -> 11.1, of which 1.3 allocates the result and 3.7 is the
+# library call with its launch.
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream=None, device=None):
     if stream is not None:
-        return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else stream)
+        return stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
     if device is not None and device.type == "cuda":
-        return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
-    return ctypes.c_void_p(0)
+        if _raw_stream is not None and device.index is not None:
+            return _raw_stream(device.index)
+        return torch.cuda.current_stream(device).cuda_stream
+    return 0
 
 
 def _check4(t, name):
     if t is None:
         return
-    if t.dtype != torch.float32 or t.dim() != 2 or t.shape[1] != 4 or not t.is_contiguous():
+    if t.dtype is not torch.float32 or t.dim() != 2 or t.size(1) != 4 or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous float32 (n, 4) tensor")
 
 
