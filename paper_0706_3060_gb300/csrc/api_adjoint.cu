@@ -394,9 +394,11 @@ int vjp_once(const float4 *pos, const float4 *prm, const float4 *lam, float4 *gr
   f.type_ends = type_ends;
   if (sc.tri) {
     f.tri = sc.geom;
-    NB_CUDA(launch_kernel(vjp_finalize_kernel<4>, sc.nblk, 256, 0, s, true, f));
+    NB_CUDA(launch_kernel(ljc ? vjp_finalize_kernel<4, true> : vjp_finalize_kernel<4, false>,
+                          sc.nblk, 256, 0, s, true, f));
   } else {
-    NB_CUDA(launch_kernel(vjp_finalize_kernel<1>, sc.nblk, 256, 0, s, true, f));
+    NB_CUDA(launch_kernel(ljc ? vjp_finalize_kernel<1, true> : vjp_finalize_kernel<1, false>,
+                          sc.nblk, 256, 0, s, true, f));
   }
   return NBODY_OK;
 }

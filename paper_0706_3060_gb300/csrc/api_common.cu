@@ -425,11 +425,13 @@ bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out) {
   const TriGeom g = tri_geom(int(n), d->h, sms * d->per_sm);
   const int slots = g.nb + tri_max_row_shares(g);
   const double bytes = double(slots) * double(n) * sizeof(float4);
-  // Softened gravity from 65536 particles stays with the block-pair tiles, whose
+  // Softened gravity from 114688 particles stays with the block-pair tiles, whose
   // partials are added exactly in fixed point with integer atomics (64 bytes a
-  // particle): as fast there (steps at 65536: 1162 us against 1167, at 262144 17.72 ms
-  // against 17.8), where the slots would grow as n^2 (134 MB and 2.1 GB).
-  if (law == NBODY_LAW_GRAV && atomic_ok && n >= 65536) return false;
+  // particle), where the slots grow as n^2 (134 MB at 65536, 0.4 GB at 114688) and the
+  // finalize with them: steps, us, here / there, 1145 / 1166 at 65536, 2554 / 2577 at
+  // 98304, 4524 / 4496 at 131072; forces with potential 1305 / 1462, 2911 / 3236, 5156 /
+  // 5575.
+  if (law == NBODY_LAW_GRAV && atomic_ok && n >= 114688) return false;
   if (bytes > sym_part_cap()) return false;
   out->tile = &kNoTile;
   out->tri = d;

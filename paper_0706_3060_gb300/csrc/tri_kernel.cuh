@@ -24,9 +24,9 @@
 // are resident from the start (taken from a queue in smaller pieces instead, 3 to 6%
 // more: 82 us against 77.5 at 16384, 298 against 287 at 32768). Two CTAs of four warps
 // per SM: one of eight, whose warps keep step with each other, took 5% longer.
-// Leapfrog steps inside a call (us), block-pair tile -> here: gravity 36.4 -> 28.2 at
-// 8192, 91.8 -> 81.9 at 16384, 308 -> 295 at 32768; LJC 44.9 -> 37.1, 129.6 -> 117.3,
-// 475 -> 444, and 1831 -> 1738 at 65536 (80% of the FP32 lane peak).
+// Leapfrog steps inside a call (us), block-pair tile -> here: gravity 36.4 -> 27.5 at
+// 8192, 91.8 -> 80.1 at 16384, 308 -> 294 at 32768; LJC 44.9 -> 36.2, 129.6 -> 116.9,
+// 475 -> 441, and 1831 -> 1721 at 65536 (80% of the FP32 lane peak).
 //
 // Sums. A target's sum is plain FP32 over at most 128 sources, then over at most four
 // such sums of a window of 64 groups, then over the four warps, each in order, and over

@@ -8,9 +8,11 @@
 // 47.2 us against 44.3 at 8192, 163 against 162 at 16384, 635 against 629 at 32768), rows
 // of 128 move the sources twice as often (LJC VJP: 1153 us at 32768 against 1065).
 // Per step with the finalize, against the block-pair tiles (us):
-//   Hermite 8192 46.6 / 79.2, 16384 163 / 215, 32768 629 / 685
-//   gravity reverse step 4096 20.8 / 27.4, 8192 47.9 / 61.7, 16384 167 / 185
-//   LJC reverse step 4096 33.1 / 46.3, 8192 78.4 / 105, 32768 1082 / 2186
+//   Hermite 8192 45.8 / 79.2, 16384 161 / 215, 32768 616 / 685
+//   gravity reverse step 4096 20.0 / 27.4, 8192 47.3 / 61.7, 16384 166 / 185
+//   LJC reverse step 4096 32.5 / 46.3, 8192 77.6 / 105, 32768 1077 / 2186
+// The next group's sources are on their way in all but jerk (600 us at 32768 without,
+// 609 with).
 #include "api_common.h"
 #include "direct_impl.h"
 #include "tri_impl.h"
@@ -27,7 +29,7 @@ cudaError_t tri_one(const TriArgs &a, bool, bool, cudaStream_t s) {
 }  // namespace
 
 const TriDesc *tri_vjp(int table) {
-  static const TriDesc jerk{4, 2, &tri_one<TriJerk, 4, true>};
+  static const TriDesc jerk{4, 2, &tri_one<TriJerk, 4, false>};
   static const TriDesc grav{4, 2, &tri_one<TriGravVjp, 4, true>};
   static const TriDesc ljc{4, 2, &tri_one<TriLjcVjp<false>, 4, true>};
   static const TriDesc ljclin{4, 2, &tri_one<TriLjcVjp<true>, 4, true>};

@@ -120,7 +120,8 @@ __device__ __forceinline__ bool tri_slot_sums(const float4 *part, long long stri
 
 // SPLIT 1: the partials of the tile and direct kernels, 256 particles per block; SPLIT 4:
 // those of the streamed triangle kernels, 64 particles per block.
-template <int SPLIT>
+// LJ: an LJC law (two rows of sums).
+template <int SPLIT, bool LJ>
 __global__ void __launch_bounds__(256) vjp_finalize_kernel(
     const __grid_constant__ VjpFinalizeArgs f) {
   if (SPLIT > 1) griddep_launch();
@@ -132,6 +133,16 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(
   double my_sigma = 0.0, my_eps = 0.0;
   float4 hA, oA, hB, oB;
   bool mine = true;
+  // SPLIT > 1: the particle's state, on its way with the slots
+  float4 x0, u0, g0 = make_float4(0.f, 0.f, 0.f, 0.f), v0 = g0;
+  if (SPLIT > 1 && run_of == 0 && i < f.n) {
+    if (LJ) {
+      x0 = f.pos[i];
+      u0 = f.lam[i];
+    }
+    if (f.accumulate) g0 = f.grad_x[i];
+    if (f.lam_v) v0 = f.lam_v[i];
+  }
   if constexpr (SPLIT > 1)
     mine = tri_slot_sums<SPLIT>(f.part_hi, f.stride, f.bstride, f.tri,
                                 f.law != NBODY_LAW_GRAV, i, run_of, hA, oA, hB, oB);
@@ -139,7 +150,7 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(
     // part_lo == nullptr: partials without low parts (Newton-symmetric gravity tiles)
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     if (SPLIT == 1) hA = oA = hB = oB = zero;
-    const bool lj = (f.law == NBODY_LAW_LJC || f.law == NBODY_LAW_LJC_LINEAR);
+    constexpr bool lj = LJ;
     const int sp = f.sym_split > 1 ? f.sym_split : 1;
     const int own_b = sp > 1 ? i / f.sym_block : 0;
     const int own_s = sp > 1 ? ((i - own_b * f.sym_block) >> 1) / (f.sym_block / 2 / sp) : 0;
@@ -207,8 +218,8 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(
       gz = f.G * az;
       gm = -f.G * aw;
     } else {
-      const float4 x = f.pos[i];
-      float4 u = f.lam[i];
+      const float4 x = SPLIT > 1 ? x0 : f.pos[i];
+      float4 u = SPLIT > 1 ? u0 : f.lam[i];
       if (!f.lam_is_u) {
         const float inv = 1.0f / x.w;
         u = make_float4(u.x * inv, u.y * inv, u.z * inv, 0.0f);
@@ -231,7 +242,8 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(
         my_eps = double(bw) * r;
       }
     }
-    float4 gxo = f.accumulate ? f.grad_x[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 gxo = g0;
+    if (SPLIT == 1 && f.accumulate) gxo = f.grad_x[i];
     gxo.x = fmaf(f.alpha, gx, gxo.x);
     gxo.y = fmaf(f.alpha, gy, gxo.y);
     gxo.z = fmaf(f.alpha, gz, gxo.z);
@@ -242,7 +254,7 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(
       f.grad_m[i] = fmaf(f.alpha, gm, gmo);
     }
     if (f.lam_v) {
-      float4 v = f.lam_v[i];
+      float4 v = SPLIT > 1 ? v0 : f.lam_v[i];
       v.x = fmaf(f.dt_next, gxo.x, v.x);
       v.y = fmaf(f.dt_next, gxo.y, v.y);
       v.z = fmaf(f.dt_next, gxo.z, v.z);
@@ -343,6 +355,13 @@ __global__ void __launch_bounds__(256) gaj_finalize_kernel(
   const int run_of = SPLIT > 1 ? threadIdx.x / kParts : 0;
   const int i = blockIdx.x * kParts + threadIdx.x - run_of * kParts;
   float4 hA, oA, hB, oB;
+  float4 x, v, a, j;  // corrector: the step's start, on its way with the slots
+  if (f.pos && run_of == 0 && i < f.n) {
+    x = f.pos[i];
+    v = f.vel[i];
+    a = f.acc[i];
+    j = f.jerk[i];
+  }
   if constexpr (SPLIT > 1) {
     if (!tri_slot_sums<SPLIT>(f.part_hi, f.stride, f.bstride, f.tri, true, i, run_of, hA, oA, hB,
                               oB))
@@ -391,7 +410,6 @@ __global__ void __launch_bounds__(256) gaj_finalize_kernel(
     // Hermite corrector (time-symmetric form):
     //   v1 = v + dt/2 (a + a1) + dt^2/12 (j - j1),
     //   x1 = x + dt/2 (v + v1) + dt^2/12 (a - a1)
-    const float4 x = f.pos[i], v = f.vel[i], a = f.acc[i], j = f.jerk[i];
     const float h = 0.5f * f.dt, q = f.dt * f.dt * (1.0f / 12.0f);
     float4 v1, x1;
     v1.x = fmaf(q, j.x - j1.x, fmaf(h, a.x + a1.x, v.x));
