@@ -50,7 +50,7 @@ constexpr int kTriWarps = 4;
 constexpr int kTriThreads = 32 * kTriWarps;
 constexpr int kTriChunk = 16;  // groups summed in registers: 128 sources for each warp
 constexpr int kTriWindow = 4;  // chunks between sums over the four warps
-constexpr int kTriLeft = 6;    // left-over groups of a window: three own, three beyond
+constexpr int kTriLeft = 3;    // left-over groups beyond the row of a window
 
 struct TriArgs {
   const float4 *p0;  // (x, y, z, m)

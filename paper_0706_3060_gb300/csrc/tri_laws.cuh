@@ -5,12 +5,12 @@
 // A law gives the words of a particle (kWords: as a target two particles' words are
 // packed in float2, as a source they are broadcast to both halves), the number of
 // sums per particle (kSums) and the pair function
-//   pair<MASK, SRC>(S, T, A, J, e2, k0, k1, both)
+//   pair<MASK, SRC>(S, T, A, J, e2, k0, k1)
 // which adds the target-side terms of both targets to A and the source-side terms to
 // J (the even target's to J[2 c], the odd target's to J[2 c + 1]). MASK: a half counts
-// only when its k0 / k1 is set, and the source side only with `both`. kFlip bit c: the
-// source-side term of sum c has the opposite sign (Newton's third law), applied when J
-// is stored. SRC false: the target side alone (direct_kernel.cuh).
+// only when its k0 / k1 is set. SRC false: the target side alone (a row's own groups,
+// direct_kernel.cuh). kFlip bit c: the source-side term of sum c has the opposite sign
+// (Newton's third law), applied when J is stored.
 //
 // The source-side sums are plain floats updated with scalar fused multiply-adds: they
 // are added up and handed from lane to lane one word at a time (tri_kernel.cuh), and
@@ -33,10 +33,6 @@ __device__ __forceinline__ float2 rsqrt2(float2 s, bool precise) {
     y = __fmul2_rn(y, __ffma2_rn(hs, __fmul2_rn(y, y), bcast(1.5f)));
   }
   return y;
-}
-
-__device__ __forceinline__ float2 only(float2 v, bool keep) {
-  return make_float2(keep ? v.x : 0.0f, keep ? v.y : 0.0f);
 }
 
 // J[0], J[1] += w * d, half by half.
@@ -73,8 +69,7 @@ struct TriGrav {
   template <bool MASK, bool SRC = true>
   static __device__ __forceinline__ void pair(const float (&S)[kWords], const float2 (&T)[kWords],
                                               float2 (&A)[kSums], float (&J)[2 * kSums],
-                                              float2 e2, bool k0 = true, bool k1 = true,
-                                              bool both = true) {
+                                              float2 e2, bool k0 = true, bool k1 = true) {
     const float2 dx = __fadd2_rn(bcast(S[0]), T[0]);
     const float2 dy = __fadd2_rn(bcast(S[1]), T[1]);
     const float2 dz = __fadd2_rn(bcast(S[2]), T[2]);
@@ -94,11 +89,10 @@ struct TriGrav {
     if (POT) A[kSums - 1] = __ffma2_rn(bcast(S[3]), y, A[kSums - 1]);
     if (!SRC) return;
     float2 wj = __fmul2_rn(T[3], y3);  // target mass: pull on the source
-    if (MASK) wj = only(wj, both);
     jfma(J, wj, dx);
     jfma(J + 2, wj, dy);
     jfma(J + 4, wj, dz);
-    if (POT) jfma(J + 2 * (kSums - 1), T[3], MASK ? only(y, both) : y);
+    if (POT) jfma(J + 2 * (kSums - 1), T[3], y);
   }
 };
 
@@ -128,8 +122,7 @@ struct TriLjc {
   template <bool MASK, bool SRC = true>
   static __device__ __forceinline__ void pair(const float (&S)[kWords], const float2 (&T)[kWords],
                                               float2 (&A)[kSums], float (&J)[2 * kSums], float2,
-                                              bool k0 = true, bool k1 = true,
-                                              bool both = true) {
+                                              bool k0 = true, bool k1 = true) {
     const float2 dx = __fadd2_rn(bcast(S[0]), T[0]);
     const float2 dy = __fadd2_rn(bcast(S[1]), T[1]);
     const float2 dz = __fadd2_rn(bcast(S[2]), T[2]);
@@ -155,7 +148,7 @@ struct TriLjc {
     A[1] = __ffma2_rn(f, dy, A[1]);
     A[2] = __ffma2_rn(f, dz, A[2]);
     if (SRC) {
-      const float2 fj = MASK ? only(f, both) : f;
+      const float2 fj = f;
       jfma(J, fj, dx);
       jfma(J + 2, fj, dy);
       jfma(J + 4, fj, dz);
@@ -164,7 +157,7 @@ struct TriLjc {
       float2 e = __fmul2_rn(qq, LIN ? y2 : y);
       e = __ffma2_rn(__fmul2_rn(ee, bcast(1.0f / 6.0f)), __ffma2_rn(u, u, neg2(u)), e);
       A[kSums - 1] = __fadd2_rn(A[kSums - 1], e);
-      if (SRC) jadd(J + 2 * (kSums - 1), MASK ? only(e, both) : e);
+      if (SRC) jadd(J + 2 * (kSums - 1), e);
     }
   }
 };

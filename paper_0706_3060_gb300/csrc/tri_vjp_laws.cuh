@@ -41,8 +41,7 @@ struct TriJerk {
   template <bool MASK, bool SRC = true>
   static __device__ __forceinline__ void pair(const float (&S)[kWords], const float2 (&T)[kWords],
                                               float2 (&A)[kSums], float (&J)[2 * kSums],
-                                              float2 e2, bool k0 = true, bool k1 = true,
-                                              bool both = true) {
+                                              float2 e2, bool k0 = true, bool k1 = true) {
     const float2 dx = __fadd2_rn(bcast(S[0]), T[0]);
     const float2 dy = __fadd2_rn(bcast(S[1]), T[1]);
     const float2 dz = __fadd2_rn(bcast(S[2]), T[2]);
@@ -73,7 +72,6 @@ struct TriJerk {
     A[5] = __ffma2_rn(wi, tz, A[5]);
     if (!SRC) return;
     float2 wj = __fmul2_rn(T[3], y3);
-    if (MASK) wj = only(wj, both);
     jfma(J, wj, dx);
     jfma(J + 2, wj, dy);
     jfma(J + 4, wj, dz);
@@ -102,8 +100,7 @@ struct TriGravVjp {
   template <bool MASK, bool SRC = true>
   static __device__ __forceinline__ void pair(const float (&S)[kWords], const float2 (&T)[kWords],
                                               float2 (&A)[kSums], float (&J)[2 * kSums],
-                                              float2 e2, bool k0 = true, bool k1 = true,
-                                              bool both = true) {
+                                              float2 e2, bool k0 = true, bool k1 = true) {
     const float2 dx = __fadd2_rn(bcast(S[0]), T[0]);
     const float2 dy = __fadd2_rn(bcast(S[1]), T[1]);
     const float2 dz = __fadd2_rn(bcast(S[2]), T[2]);
@@ -134,7 +131,7 @@ struct TriGravVjp {
     A[2] = __ffma2_rn(y3, vz, A[2]);
     A[3] = __ffma2_rn(lj, y3, A[3]);
     if (!SRC) return;
-    const float2 yj = MASK ? only(y3, both) : y3;
+    const float2 yj = y3;
     jfma(J, yj, vx);
     jfma(J + 2, yj, vy);
     jfma(J + 4, yj, vz);
@@ -176,8 +173,7 @@ struct TriLjcVjp {
   template <bool MASK, bool SRC = true>
   static __device__ __forceinline__ void pair(const float (&S)[kWords], const float2 (&T)[kWords],
                                               float2 (&A)[kSums], float (&J)[2 * kSums], float2,
-                                              bool k0 = true, bool k1 = true,
-                                              bool both = true) {
+                                              bool k0 = true, bool k1 = true) {
     const float2 dx = __fadd2_rn(bcast(S[0]), T[0]);
     const float2 dy = __fadd2_rn(bcast(S[1]), T[1]);
     const float2 dz = __fadd2_rn(bcast(S[2]), T[2]);
@@ -223,8 +219,8 @@ struct TriLjcVjp {
     A[6] = __ffma2_rn(phi, dz, A[6]);
     A[7] = __ffma2_rn(dw, phi_lj, A[7]);
     if (!SRC) return;
-    const float2 cj = MASK ? only(c, both) : c, pj = MASK ? only(phi, both) : phi;
-    const float2 dj = MASK ? only(dw, both) : dw;
+    const float2 cj = c, pj = phi;
+    const float2 dj = dw;
     jfma(J, pj, wx);
     jfma(J, cj, dx);
     jfma(J + 2, pj, wy);
