@@ -12,6 +12,12 @@
 // direct_kernel.cuh). kFlip bit c: the source-side term of sum c has the opposite sign
 // (Newton's third law), applied when J is stored.
 //
+// The particles' words are read with ordinary loads: the finalize in front of these
+// kernels lets them be placed early (griddep_launch) and writes positions, velocities and
+// lambda while they are, and only ordinary loads are ordered by griddep_start; the
+// non-coherent ones (__ldg) want memory that nobody writes as long as the kernel lives.
+// Parameters are written by no kernel of a chain.
+//
 // The source-side sums are plain floats updated with scalar fused multiply-adds: they
 // are added up and handed from lane to lane one word at a time (tri_kernel.cuh), and
 // with three register operands the packed instruction loses time to register banks
@@ -54,7 +60,7 @@ struct TriGrav {
   // words of particle i, or of the massless pad far away
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *, const float4 *,
                                               int i, int n, float (&w)[kWords]) {
-    const float4 p = i < n ? __ldg(p0 + i) : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
     w[0] = p.x;
     w[1] = p.y;
     w[2] = p.z;
@@ -105,7 +111,7 @@ struct TriLjc {
   static constexpr unsigned kFlip = 0x7;
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *p1, const float4 *,
                                               int i, int n, float (&w)[kWords]) {
-    const float4 p = i < n ? __ldg(p0 + i) : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
     const float4 q = i < n ? __ldg(p1 + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     w[0] = p.x;
     w[1] = p.y;

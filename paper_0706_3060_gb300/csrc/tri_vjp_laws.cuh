@@ -11,8 +11,8 @@ namespace nbody {
 // Words x, y, z, m of particle i and three more from its element of `p2`.
 __device__ __forceinline__ void load_pos_and(const float4 *p0, const float4 *p2, int i, int n,
                                              float (&w)[7]) {
-  const float4 p = i < n ? __ldg(p0 + i) : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
-  const float4 v = i < n ? __ldg(p2 + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+  const float4 v = i < n ? p2[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   w[0] = p.x;
   w[1] = p.y;
   w[2] = p.z;
@@ -151,9 +151,9 @@ struct TriLjcVjp {
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *p1,
                                               const float4 *p2, int i, int n,
                                               float (&w)[kWords]) {
-    const float4 p = i < n ? __ldg(p0 + i) : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
     const float4 q = i < n ? __ldg(p1 + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    const float4 l = i < n ? __ldg(p2 + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float4 l = i < n ? p2[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     const float inv = i < n ? 1.0f / p.w : 0.0f;
     w[0] = p.x;
     w[1] = p.y;
