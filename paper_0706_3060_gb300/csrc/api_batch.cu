@@ -34,6 +34,7 @@ struct nbody_batch_plan {
   int *d_sys_of = nullptr;
   int *d_counter = nullptr;  // one counter per force evaluation of a run
   int counters = 0;
+  std::vector<int *> old_counters;  // outgrown ones, which captured graphs may still use
   float4 *d_part = nullptr;  // [2][max_slices][total]
   // packed tiles: per-law pair buffers and, per system, (offset, pair base, n, law)
   float4 *d_jgrav = nullptr;
@@ -59,6 +60,7 @@ void free_plan(nbody_batch_plan *p) {
   cudaFree(p->d_sys);
   cudaFree(p->d_sys_of);
   cudaFree(p->d_counter);
+  for (int *c : p->old_counters) cudaFree(c);
   cudaFree(p->d_part);
   cudaFree(p->d_jgrav);
   cudaFree(p->d_jljc);
@@ -66,12 +68,18 @@ void free_plan(nbody_batch_plan *p) {
   delete p;
 }
 
+// At least `need` counters. The plan's graph, or one that the caller captured, holds the
+// address of the counters of its own run: outgrown ones live as long as the plan (they at
+// least double each time, so all of them take less than the newest).
 int ensure_counters(nbody_batch_plan *p, int need) {
   if (p->counters >= need) return NBODY_OK;
-  if (p->d_counter) NB_CUDA(cudaFree(p->d_counter));
-  p->d_counter = nullptr;
-  NB_CUDA(cudaMalloc(&p->d_counter, sizeof(int) * size_t(need)));
-  p->counters = need;
+  const int64_t twice = std::min<int64_t>(2 * int64_t(p->counters), INT32_MAX);
+  const int count = int(std::max<int64_t>(need, twice));
+  int *fresh = nullptr;
+  NB_CUDA(cudaMalloc(&fresh, sizeof(int) * size_t(count)));
+  if (p->d_counter) p->old_counters.push_back(p->d_counter);
+  p->d_counter = fresh;
+  p->counters = count;
   return NBODY_OK;
 }
 
