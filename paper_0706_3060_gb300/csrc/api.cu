@@ -195,6 +195,7 @@ int eval_and_finalize(const float4 *pos, const float4 *prm, const nbody_params &
   const bool prep = prepare_next && plan.tile->packed && (f.mode & kFinKickDrift);
   f.jnext = prep ? sc.jbuf : nullptr;
   f.tri = plan.tri ? plan.geom : TriGeom{};
+  f.tri.low = pot && plan.tri && plan.tri->low;
   f.jn_block = plan.tile->sym ? plan.tile->tile_i : 0;
   f.jn_words = p.law == NBODY_LAW_GRAV ? 2 : 3;
   f.rezero = (prep && plan.atomic) ? 1 : 0;

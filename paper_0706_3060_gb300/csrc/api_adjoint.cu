@@ -76,7 +76,7 @@ int vjp_untiled(int law, int n, int sms, cudaStream_t s, VjpScratch *sc, size_t 
   int slots = 1;
   if (n > 16 * sms) {
     if (n > 0x7fffffff - 64 * 64) return NBODY_OK;
-    sc->tri = tri_vjp(sc->table);
+    sc->tri = tri_vjp(sc->table, n);
     sc->geom = tri_geom(n, sc->tri->h, sms * sc->tri->per_sm);
     slots = sc->geom.nb + tri_max_row_shares(sc->geom);
     if (double(blocks) * slots * n * sizeof(float4) > sym_part_cap()) {

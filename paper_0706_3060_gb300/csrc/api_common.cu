@@ -423,7 +423,7 @@ bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out) {
                      : law == NBODY_LAW_LJC ? tri_ljc(n)
                                             : tri_ljclin(n);
   const TriGeom g = tri_geom(int(n), d->h, sms * d->per_sm);
-  const int slots = g.nb + tri_max_row_shares(g);
+  const int slots = tri_slots(g);
   const double bytes = double(slots) * double(n) * sizeof(float4);
   // Softened gravity from 114688 particles stays with the block-pair tiles, whose
   // partials are added exactly in fixed point with integer atomics (64 bytes a

@@ -125,6 +125,19 @@ __global__ void __launch_bounds__(kFinThreads * SPLIT) finalize_kernel(
       // the source-side slots 0 .. row - 1, then the target-side slots from nb on
       run(k0, min(k1, below) - k0, 1);
       run(f.tri.nb + max(k0, below) - below, k1 - max(k0, below), 1);
+    if (f.tri.low && !plain) {  // gravity's potential: the low parts of the target-side ones
+      const float *low = reinterpret_cast<const float *>(
+          f.part_hi + (long long)(f.tri.nb + tri_max_row_shares(f.tri)) * f.stride);
+      const int end = k1 - below;
+      for (int k = max(k0, below) - below; k < end; k += 4) {
+        float l[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) l[u] = low[(long long)min(k + u, end - 1) * f.stride + i];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k + u < end) lo.w = __fadd_rn(lo.w, l[u]);
+      }
+    }
     }
     const int at = threadIdx.x - run_of * kFinThreads;
     if (run_of > 0) {

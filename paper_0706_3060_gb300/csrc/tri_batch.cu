@@ -12,7 +12,7 @@ template <bool PRECISE>
 cudaError_t go(const TriBatchArgs &a, cudaStream_t s) {
   auto k = tri_batch_kernel<PRECISE>;
   constexpr size_t kSmem =
-      std::max(TriTile<TriGrav<false, PRECISE>, kTriBatchGrav>::kSmemBytes,
+      std::max(TriTile<TriGrav<false, PRECISE, false>, kTriBatchGrav>::kSmemBytes,
                TriTile<TriLjc<false, false, PRECISE>, kTriBatchLjc>::kSmemBytes);
   static std::atomic<bool> opted[kMaxDevicesTile];
   int dev = 0;

@@ -49,14 +49,14 @@ __global__ void __launch_bounds__(kTriThreads, 2) tri_batch_kernel(
     t.eps2 = g.eps2;
     t.geom.n = g.n;
     if (g.law == 0)
-      tri_run<TriGrav<false, PRECISE>, kTriBatchGrav, true>(t, g.row, g.d0, g.d1, g.o0, g.o1,
-                                                            g.slot, tri_smem);
+      tri_run<TriGrav<false, PRECISE, false>, kTriBatchGrav, true>(t, g.row, g.d0, g.d1, g.o0, g.o1,
+                                                            g.slot, nullptr, tri_smem);
     else if (g.law == 1)
       tri_run<TriLjc<false, false, PRECISE>, kTriBatchLjc, true>(t, g.row, g.d0, g.d1, g.o0, g.o1,
-                                                                 g.slot, tri_smem);
+                                                                 g.slot, nullptr, tri_smem);
     else
       tri_run<TriLjc<true, false, PRECISE>, kTriBatchLjc, true>(t, g.row, g.d0, g.d1, g.o0, g.o1,
-                                                                g.slot, tri_smem);
+                                                                g.slot, nullptr, tri_smem);
     if (threadIdx.x == 0) next = mine;
     __syncthreads();
     s = next;

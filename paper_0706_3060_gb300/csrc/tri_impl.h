@@ -32,7 +32,7 @@ struct TriImpl {
     return precise ? tri_go<LAW<false, true>, H, MINB, AHEAD>(a, s)
                    : tri_go<LAW<false, false>, H, MINB, AHEAD>(a, s);
   }
-  static TriDesc desc() { return TriDesc{H, MINB, &launch}; }
+  static TriDesc desc() { return TriDesc{H, MINB, LAW<true, false>::kLow, &launch}; }
 };
 
 }  // namespace nbody

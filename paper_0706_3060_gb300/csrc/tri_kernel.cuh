@@ -28,10 +28,20 @@
 // 8192, 91.8 -> 80.1 at 16384, 308 -> 294 at 32768; LJC 44.9 -> 36.2, 129.6 -> 116.9,
 // 475 -> 441, and 1831 -> 1721 at 65536 (80% of the FP32 lane peak).
 //
-// Sums. A target's sum is plain FP32 over at most 128 sources, then over at most four
-// such sums of a window of 64 groups, then over the four warps, each in order, and over
-// the windows of a share with TwoSum. A source's sum is plain FP32 over the 2 H targets
-// of a step and then over the steps. Partials go, per row b,
+// Sums. A target's sum is plain FP32 over the sources that one warp meets in kChunk groups
+// (128 with 16 groups, and the left-over ones), then over at most four such sums (a
+// window), then over the four warps, each in order, and over the windows of a share with
+// TwoSum. A source's sum is plain FP32 over the 2 H targets of a step and over 32 / kParts
+// steps, then over the parts. Laws with kFine (gravity's forces from 8192 particles on, its
+// VJP of 4096 to 8191), where the tiles are nearer to the 64-bit values than the longer
+// sums, take 8 or 4 groups, 2 or 4 parts and TwoSum over the warps, and their potentials
+// keep the low part of a share's sum. Rms errors against 64 bits, plain / fine / tile:
+// potential 2.87e-8 / 2.54e-8 / 2.55e-8 at 12287, 2.65e-8 / 2.42e-8 / 2.48e-8 at 65536;
+// accelerations 5.1e-8 / 4.6e-8 / 4.8e-8 at 12287; VJP, mass terms, 1.89e-7 / 1.61e-7 /
+// 1.70e-7 at 6500. Leapfrog steps (us), plain / fine: 27.8 / 28.4 at 8192, 80.4 / 80.7 at
+// 16384, 1143.9 / 1143.8 at 65536, with potential 772 / 782 at 50021; reverse steps 25.2 /
+// 25.7 at 5000. The LJC laws' errors are those of their pair terms (forces 8e-7 either way).
+// Partials go, per row b,
 //   * source side: one per row and particle beyond it, to slot b;
 //   * target side: one per share and target, to slot nb + (share - first share of
 //     the row);
@@ -48,8 +58,7 @@ namespace nbody {
 
 constexpr int kTriWarps = 4;
 constexpr int kTriThreads = 32 * kTriWarps;
-constexpr int kTriChunk = 16;  // groups summed in registers: 128 sources for each warp
-constexpr int kTriWindow = 4;  // chunks between sums over the four warps
+constexpr int kTriWindow = 4;  // chunks (L::kChunk groups) between sums over the four warps
 constexpr int kTriLeft = 3;    // left-over groups beyond the row of a window
 
 struct TriArgs {
@@ -76,6 +85,13 @@ struct TriTile {
   static_assert(kTriWarps * L::kSums >= L::kWords, "the target words are staged in the sums' place");
 };
 
+// Low parts of the fourth target-side sums that share `k` of a row leaves: a float for each
+// particle, behind the slots.
+__device__ __forceinline__ float *tri_low(const TriArgs &a, int k) {
+  const int slot = a.geom.nb + tri_max_row_shares(a.geom);
+  return reinterpret_cast<float *>(a.part + (long long)slot * a.stride) + (long long)k * a.stride;
+}
+
 // Place of a row's t-th target in an array of the row: the two targets of an f32x2
 // value next to each other, lanes in order.
 __device__ __forceinline__ int tri_place(int t) {
@@ -100,7 +116,7 @@ __device__ __forceinline__ void tri_store(const TriArgs &a, int slot, int i,
 // return B holds the source-side sums of source (lane + s0 + STEPS) & 31 over these steps,
 // before their sign change.
 template <class L, int H, int STEPS>
-__device__ __forceinline__ void tri_group(float eps2, const float2 (&T)[H][L::kWords],
+__device__ __forceinline__ void tri_steps(float eps2, const float2 (&T)[H][L::kWords],
                                           float2 (&A)[H][L::kSums], float (&B)[L::kSums],
                                           float (&S)[L::kWords]) {
   const int next = (threadIdx.x & 31) + 1;
@@ -119,6 +135,29 @@ __device__ __forceinline__ void tri_group(float eps2, const float2 (&T)[H][L::kW
       B[c] = __shfl_sync(0xffffffffu, B[c] + (J[2 * c] + J[2 * c + 1]), next);
 #pragma unroll
     for (int c = 0; c < L::kWords; ++c) S[c] = __shfl_sync(0xffffffffu, S[c], next);
+  }
+}
+
+// All 32 steps from the lane's own source on, in L::kParts parts: each part's sums are added
+// to the earlier ones' as the source moves on.
+template <class L, int H>
+__device__ __forceinline__ void tri_group(float eps2, const float2 (&T)[H][L::kWords],
+                                          float2 (&A)[H][L::kSums], float (&B)[L::kSums],
+                                          float (&S)[L::kWords]) {
+  constexpr int kSteps = 32 / L::kParts;
+  if constexpr (L::kParts == 1) {
+    tri_steps<L, H, 32>(eps2, T, A, B, S);
+  } else {
+    const int from = (threadIdx.x & 31) + kSteps;
+#pragma unroll
+    for (int c = 0; c < L::kSums; ++c) B[c] = 0.0f;
+#pragma unroll 1
+    for (int k = 0; k < L::kParts; ++k) {
+      float part[L::kSums];
+      tri_steps<L, H, kSteps>(eps2, T, A, part, S);
+#pragma unroll
+      for (int c = 0; c < L::kSums; ++c) B[c] = __shfl_sync(0xffffffffu, B[c], from) + part[c];
+    }
   }
 }
 
@@ -152,7 +191,7 @@ __device__ __forceinline__ void tri_own_group(float eps2, int own, int s0,
 // then the groups o0 .. o1-1 beyond the row (counted from the first beyond).
 template <class L, int H, bool AHEAD>
 __device__ __forceinline__ void tri_run(const TriArgs &a, int row, int d0, int d1, int o0, int o1,
-                                        int target_slot, float *smem) {
+                                        int target_slot, float *low, float *smem) {
   using T_ = TriTile<L, H>;
   constexpr int R = T_::kRow, NS = L::kSums;
   float *red = smem;             // [warp][sum][R]
@@ -189,33 +228,39 @@ __device__ __forceinline__ void tri_run(const TriArgs &a, int row, int d0, int d
   // the window's target sums of the four warps into comp, or out when nothing follows,
   // and its left-over groups' source-side sums
   auto close_window = [&](bool done) {
-    float v[NS];
+    float v[NS], l[NS];
     __syncthreads();
     for (int t = tid; t < R; t += kTriThreads) {
       const int at = tri_place(t), i = row * R + t;
 #pragma unroll
       for (int c = 0; c < NS; ++c) {
         v[c] = red[c * R + at];
+        l[c] = 0.0f;
 #pragma unroll
-        for (int w = 1; w < kTriWarps; ++w) v[c] += red[(w * NS + c) * R + at];
-      }
-      if (folded) {
-#pragma unroll
-        for (int c = 0; c < NS; ++c) {
-          float hi = comp[c * R + t], lo = comp[(NS + c) * R + t];
-          comp_add(hi, lo, v[c]);
-          comp[c * R + t] = hi;
-          comp[(NS + c) * R + t] = lo;
-          v[c] = hi + lo;
+        for (int w = 1; w < kTriWarps; ++w) {
+          const float s = red[(w * NS + c) * R + at];
+          if (L::kFine) comp_add(v[c], l[c], s);
+          else v[c] += s;
         }
-      } else if (!done) {
-#pragma unroll
-        for (int c = 0; c < NS; ++c) {
+        if (folded) {
+          l[c] += comp[(NS + c) * R + t];
+          comp_add(v[c], l[c], comp[c * R + t]);
+        }
+        if (!done) {
           comp[c * R + t] = v[c];
-          comp[(NS + c) * R + t] = 0.0f;
+          comp[(NS + c) * R + t] = l[c];
         }
       }
-      if (done && i < n) tri_store<L>(a, target_slot, i, v);
+      if (done && i < n) {
+#pragma unroll
+        for (int c = 0; c < NS; ++c) {
+          const float s = v[c] + l[c];
+          l[c] = __fsub_rn(l[c], __fsub_rn(s, v[c]));  // what s leaves out (Fast2Sum)
+          v[c] = s;
+        }
+        tri_store<L>(a, target_slot, i, v);
+        if (L::kLow) low[i] = l[NS - 1];
+      }
     }
     for (int q = warp; q < nleft; q += kTriWarps) {  // warps' parts in order
 #pragma unroll
@@ -234,8 +279,8 @@ __device__ __forceinline__ void tri_run(const TriArgs &a, int row, int d0, int d
   // groups g0 .. g1-1, all own (DIAG) or all beyond the row; `more`: others follow
   auto groups = [&](auto diag, int g0, int g1, bool more) {
     constexpr bool DIAG = decltype(diag)::value;
-    for (int g = g0; g < g1; g += kTriChunk) {
-      const int k = min(kTriChunk, g1 - g);
+    for (int g = g0; g < g1; g += L::kChunk) {
+      const int k = min(L::kChunk, g1 - g);
       const int quads = k >> 2, left = k & 3;
       float v[NS], S[L::kWords];
       auto source_sums = [&]() {
@@ -259,7 +304,7 @@ __device__ __forceinline__ void tri_run(const TriArgs &a, int row, int d0, int d
         if constexpr (DIAG) {
           tri_own_group<L, H, 32>(a.eps2, gg - 2 * H * row, 0, T, A, S);
         } else {
-          tri_group<L, H, 32>(a.eps2, T, A, v, S);
+          tri_group<L, H>(a.eps2, T, A, v, S);
           source_sums();
           if (i < n) tri_store<L>(a, row, i, v);
         }
@@ -271,7 +316,7 @@ __device__ __forceinline__ void tri_run(const TriArgs &a, int row, int d0, int d
           tri_own_group<L, H, 8>(a.eps2, gg - 2 * H * row, s0, T, A, S);
           continue;
         }
-        tri_group<L, H, 8>(a.eps2, T, A, v, S);
+        tri_steps<L, H, 8>(a.eps2, T, A, v, S);
         source_sums();
 #pragma unroll
         for (int c = 0; c < NS; ++c)
@@ -289,7 +334,7 @@ __device__ __forceinline__ void tri_run(const TriArgs &a, int row, int d0, int d
           A[r][c] = make_float2(0.0f, 0.0f);
         }
       ++chunks;
-      const bool done = !more && g + kTriChunk >= g1;
+      const bool done = !more && g + L::kChunk >= g1;
       if (done || chunks == kTriWindow) close_window(done);
     }
   };
@@ -313,7 +358,9 @@ __global__ void __launch_bounds__(kTriThreads, MINB) tri_kernel(const __grid_con
     const int d0 = tri_own(a.geom, row, p), d1 = tri_own(a.geom, row, stop);
     int first, count;
     tri_row_shares(a.geom, row, first, count);
-    tri_run<L, H, AHEAD>(a, row, d0, d1, p - d0, stop - d1, a.geom.nb + share - first, tri_smem);
+    const int k = share - first;
+    tri_run<L, H, AHEAD>(a, row, d0, d1, p - d0, stop - d1, a.geom.nb + k,
+                         L::kLow ? tri_low(a, k) : nullptr, tri_smem);
   }
 }
 

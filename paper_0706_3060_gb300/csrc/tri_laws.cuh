@@ -10,7 +10,8 @@
 // J (the even target's to J[2 c], the odd target's to J[2 c + 1]). MASK: a half counts
 // only when its k0 / k1 is set. SRC false: the target side alone (a row's own groups,
 // direct_kernel.cuh). kFlip bit c: the source-side term of sum c has the opposite sign
-// (Newton's third law), applied when J is stored.
+// (Newton's third law), applied when J is stored. kChunk, kParts: lengths of the plain sums;
+// kFine, kLow: compensated sums and the potential's low parts (tri_kernel.cuh, Sums).
 //
 // The particles' words are read with ordinary loads: the finalize in front of these
 // kernels lets them be placed early (griddep_launch) and writes positions, velocities and
@@ -52,11 +53,13 @@ __device__ __forceinline__ void jadd(float *J, float2 v) {
 }
 
 // Softened gravity (Eq. 1): words x, y, z, m; sums m y^3 d (and m y with POT).
-template <bool POT, bool PRECISE>
+template <bool POT, bool PRECISE, bool FINE>
 struct TriGrav {
   static constexpr int kWords = 4;
   static constexpr int kSums = POT ? 4 : 3;
   static constexpr unsigned kFlip = 0x7;
+  static constexpr bool kFine = FINE, kLow = FINE && POT;
+  static constexpr int kChunk = FINE ? 8 : 16, kParts = FINE ? 2 : 1;
   // words of particle i, or of the massless pad far away
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *, const float4 *,
                                               int i, int n, float (&w)[kWords]) {
@@ -109,6 +112,8 @@ struct TriLjc {
   static constexpr int kWords = 6;
   static constexpr int kSums = POT ? 4 : 3;
   static constexpr unsigned kFlip = 0x7;
+  static constexpr bool kFine = false, kLow = false;
+  static constexpr int kChunk = 16, kParts = 1;
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *p1, const float4 *,
                                               int i, int n, float (&w)[kWords]) {
     const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);

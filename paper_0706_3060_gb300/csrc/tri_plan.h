@@ -37,6 +37,7 @@ struct TriGeom {
   int nshare;  // shares
   int extra;   // cost of a row besides its units
   long long total;  // cost of the line
+  int low;     // the shares' low parts follow the slots (tri_slots)
 };
 
 // Units of row b, and how many of the first p of them are own units (the others are
@@ -59,6 +60,7 @@ NBODY_HD TriGeom tri_geom(int n, int h, int max_share) {
   t.nb = int(((long long)n + 64 * h - 1) / (64 * h));
   t.ng = int(((long long)n + kTriGroup - 1) / kTriGroup);
   t.extra = kTriRowCost;
+  t.low = 0;
   t.total = tri_row_start(t, t.nb);
   // Shares between a row's first and last must own units of it (tri_row_shares): with
   // the row cost they do when a share is longer than 2 (kTriRowCost + 1); where shares
@@ -112,6 +114,13 @@ NBODY_HD void tri_row_shares(const TriGeom &t, int b, int &first, int &count) {
 // Most shares that a row can have: rows get shorter, so row 0's length decides.
 NBODY_HD int tri_max_row_shares(const TriGeom &t) {
   return int((long long)(t.ng + t.extra) * t.nshare / t.total + 2);
+}
+
+// Slots (of a float4 for each particle) of a force evaluation: a source-side one per row,
+// target-side ones of the row with the most shares, and a float for each of the latter.
+NBODY_HD int tri_slots(const TriGeom &t) {
+  const int shares = tri_max_row_shares(t);
+  return t.nb + shares + (shares + 3) / 4;
 }
 
 }  // namespace nbody

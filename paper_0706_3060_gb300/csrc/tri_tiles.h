@@ -13,6 +13,7 @@ namespace nbody {
 struct TriDesc {
   int h;         // f32x2 register groups per thread: rows of 64 h particles
   int per_sm;    // CTAs per SM (by registers): the grid is one wave
+  bool low;      // evaluations with the potential leave its sums' low parts (kLow)
   cudaError_t (*launch)(const TriArgs &, bool pot, bool precise, cudaStream_t);
 };
 
@@ -21,6 +22,6 @@ const TriDesc *tri_grav(int64_t n);
 const TriDesc *tri_ljc(int64_t n);
 const TriDesc *tri_ljclin(int64_t n);
 // Kernel for a VJP or jerk tile table (tri_vjp.cu; no potential or precise variants).
-const TriDesc *tri_vjp(int table);
+const TriDesc *tri_vjp(int table, int64_t n);
 
 }  // namespace nbody

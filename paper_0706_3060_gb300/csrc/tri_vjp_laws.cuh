@@ -29,6 +29,8 @@ struct TriJerk {
   static constexpr int kWords = 7;
   static constexpr int kSums = 6;
   static constexpr unsigned kFlip = 0x3f;
+  static constexpr bool kFine = false, kLow = false;
+  static constexpr int kChunk = 16, kParts = 1;
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *, const float4 *p2,
                                               int i, int n, float (&w)[kWords]) {
     load_pos_and(p0, p2, i, n, w);
@@ -84,10 +86,13 @@ struct TriJerk {
 // Gravity VJP: w = m_k lam_j - m_j lam_k; the target's sums are
 // y^3 (w - 3 y^2 (d.w) d) and (lam_j.d) y^3, the source's -y^3 (w - ...) and
 // -(lam_k.d) y^3: 35 FP32 lane operations for both.
+template <bool FINE>
 struct TriGravVjp {
   static constexpr int kWords = 7;
   static constexpr int kSums = 4;
   static constexpr unsigned kFlip = 0xf;
+  static constexpr bool kFine = FINE, kLow = false;
+  static constexpr int kChunk = FINE ? 4 : 16, kParts = FINE ? 4 : 1;
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *, const float4 *p2,
                                               int i, int n, float (&w)[kWords]) {
     load_pos_and(p0, p2, i, n, w);
@@ -148,6 +153,8 @@ struct TriLjcVjp {
   static constexpr int kWords = 9;
   static constexpr int kSums = 8;
   static constexpr unsigned kFlip = 0x77;
+  static constexpr bool kFine = false, kLow = false;
+  static constexpr int kChunk = 16, kParts = 1;
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *p1,
                                               const float4 *p2, int i, int n,
                                               float (&w)[kWords]) {
