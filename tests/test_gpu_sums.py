@@ -24,7 +24,7 @@ def _compare(kinds, ref, floor=0.05):
     assert own <= SPREAD * tile, f"rms error {own:.3e}, tile {tile:.3e}"
 
 
-@pytest.mark.parametrize("n", [8192, 12287, 32769])
+@pytest.mark.parametrize("n", [4001, 8192, 12287, 32769])
 def test_forces_and_potential(n):
     nb = lib()
     g = workloads.plummer(n, seed=n, eps=0.01)
@@ -37,6 +37,22 @@ def test_forces_and_potential(n):
     _compare([o[:, :3] for o in out], ref)
     _compare([o[:, 3] for o in out], phi)
     assert torch.equal(out[0][:, :3], nb.forces(pos, eps=eps)[:, :3])
+
+
+@pytest.mark.parametrize("n", [20001, 65536])
+def test_subset(n):
+    """Four lists of 2000 active particles."""
+    nb = lib()
+    g = workloads.plummer(n, seed=n, eps=0.01)
+    pos, _ = grav_tensors(g)
+    eps = float(np.float32(g.eps))
+    x, _, m = g.f32_as_f64()
+    idx = np.random.default_rng(n).permutation(n)[:8000].astype(np.int32)
+    ref = oracle.grav_accel(x, m, eps=eps, idx=idx)
+    tile, js = nb.get_config(nb.LAW_GRAV, 2000)
+    out = [torch.cat([nb.forces_subset(pos, torch.from_numpy(k).to(dev()), eps=eps, **kw)
+                      for k in np.split(idx, 4)]) for kw in ({}, dict(tile=tile, jsplit=js))]
+    _compare([o[:, :3] for o in out], ref)
 
 
 @pytest.mark.parametrize("n", [5000, 6500])
