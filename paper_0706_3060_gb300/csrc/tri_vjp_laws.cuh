@@ -166,7 +166,9 @@ struct TriLjcVjp {
     w[1] = p.y;
     w[2] = p.z;
     w[3] = q.x;
-    w[4] = q.y;
+    // pads and atoms without a radius: k2 below is 0, and 1 / s has to be finite (kept here,
+    // once per load; a clamp in the pair function takes 1% of the kernel)
+    w[4] = q.y == 0.0f ? 1e-30f : q.y;
     w[5] = q.z;
     w[6] = -(l.x * inv);
     w[7] = -(l.y * inv);
