@@ -232,11 +232,17 @@ __global__ void __launch_bounds__(256) vjp_finalize_kernel(
       const float4 q = f.prm[i];
       const int t = int(q.w);
       if (f.type_part && t >= 0 && t < 4) {
-        // 1 / e2, e2 = (24 eps_k): the FP32 reciprocal and two Newton steps
+        // 1 / e2, e2 = (24 eps_k): the FP32 reciprocal and two Newton steps, or where that
+        // leaves FP32's range the division
         const double e2 = double(q.z) * double(q.z);
-        double r = double(1.0f / float(e2));
-        r = r * (2.0 - e2 * r);
-        r = r * (2.0 - e2 * r);
+        double r;
+        if (e2 > 1e-36 && e2 < 1e36) {
+          r = double(1.0f / float(e2));
+          r = r * (2.0 - e2 * r);
+          r = r * (2.0 - e2 * r);
+        } else {
+          r = 1.0 / e2;
+        }
         my_type = t;
         my_sigma = double(aw);
         my_eps = double(bw) * r;
