@@ -38,22 +38,37 @@ def _side_stream(dev):
 
 
 class _Cfg:
-    def __init__(self, law, dt, nsteps, k, G, eps, q=None, types=None, kq=None, ntypes=4):
+    def __init__(self, law, dt, nsteps, k, G, eps, q=None, types=None, kq=None, ntypes=4,
+                 keep_bytes=None):
         self.law, self.dt, self.nsteps, self.k = law, float(dt), int(nsteps), int(k)
+        self.keep_bytes = keep_bytes
         self.G, self.eps = float(G), float(eps)
         self.q, self.types, self.kq, self.ntypes = q, types, kq, ntypes
 
 
-def _kept_steps(n, nsteps, k, dev):
-    """Steps, counted from the last, whose positions the forward pass keeps: 16 bytes a
-    particle and step, as far as they take no more than a 256th of the device's memory or
-    than the checkpoints (80 bytes a particle and chunk) and the two chunks' positions
-    that the backward pass holds otherwise. Each step kept is a force evaluation that the
-    backward pass need not repeat (40 steps of 16384 particles, k = 10: 27 of 108
+_KEEP_ALWAYS = 32 << 20  # bytes of positions that are kept without asking what is free
+
+
+def _kept_steps(n, nsteps, k, dev, keep_bytes=None):
+    """Steps, counted from the last, whose positions the forward pass keeps (16 bytes a
+    particle and step, and once more per chunk). All of them where they take no more than
+    the checkpoints would (80 bytes a particle and chunk, and the newest chunk's positions);
+    else as many as fit in ``keep_bytes``, or without it in 32 MiB, or in a 256th of the
+    device's memory and a 64th of what is free of it, so that several graphs alive at once
+    leave each other room; always the newest chunk's. Each step kept is a force evaluation
+    that the backward pass need not repeat (40 steps of 16384 particles, k = 10: 27 of 108
     evaluations and products, 12.6 ms -> 10.3)."""
-    instead = 5 * -(-nsteps // k) + 2 * k
-    budget = torch.cuda.get_device_properties(dev).total_memory // 256
-    return max(k, instead, budget // (16 * max(n, 1)))
+    row = 16 * max(n, 1)
+    chunks = -(-nsteps // k)
+    if nsteps + chunks <= 5 * chunks + k:
+        return nsteps
+    if keep_bytes is None:
+        keep_bytes = _KEEP_ALWAYS
+        if row * (nsteps + chunks) > keep_bytes and not torch.cuda.is_current_stream_capturing():
+            free, total = torch.cuda.mem_get_info(dev)
+            free += torch.cuda.memory_reserved(dev) - torch.cuda.memory_allocated(dev)
+            keep_bytes = max(keep_bytes, min(total // 256, free // 64))
+    return max(k, keep_bytes // row * k // (k + 1))
 
 
 def _prm(cfg, sig_t, eps_t):
@@ -80,7 +95,7 @@ class NBodyLeapfrog(torch.autograd.Function):
         prm = _prm(cfg, sig_t, eps_t)
         chunks = []  # (positions, None) or (None, checkpoint) of each chunk
         done = 0
-        kept = _kept_steps(n, cfg.nsteps, cfg.k, dev)
+        kept = _kept_steps(n, cfg.nsteps, cfg.k, dev, cfg.keep_bytes)
         while done < cfg.nsteps:
             steps = min(cfg.k, cfg.nsteps - done)
             trace = ckpt = None
@@ -172,18 +187,24 @@ class NBodyLeapfrog(torch.autograd.Function):
 
 
 def leapfrog(x0, v0, m, *, dt, nsteps, k=20, G=1.0, eps=0.0, law=LAW_GRAV, q=None,
-             types=None, sig_t=None, eps_t=None, kq=None):
+             types=None, sig_t=None, eps_t=None, kq=None, keep_bytes=None):
     """Differentiable leapfrog: returns (x_T, v_T); gradients flow to x0, v0, m
     and (LJC) sig_t, eps_t. Gravity by default; pass law=LAW_LJC (or
     LAW_LJC_LINEAR, the linear dielectric) with per-atom charges q (float64),
     int32 types and per-type sig_t, eps_t for LJ + Coulomb; kq defaults to
-    k_e / 80 (constant) or k_e / 4 (linear, dielectric 4 r)."""
+    k_e / 80 (constant) or k_e / 4 (linear, dielectric 4 r).
+
+    Positions between the forward and the backward pass: those of the newest ``k`` steps and
+    as many more as fit in ``keep_bytes`` (0: no more; None: 32 MiB, or up to a 256th of the
+    device's memory and a 64th of what is free); the older chunks of k steps are recomputed
+    from checkpoints. The gradients are the same."""
     if law in _LJC_LAWS:
         if kq is None:
             kq = api.COULOMB_K / (80.0 if law == LAW_LJC else 4.0)
         ntypes = int(sig_t.shape[0])
-        cfg = _Cfg(law, dt, nsteps, k, G, eps, q=q, types=types, kq=kq, ntypes=ntypes)
+        cfg = _Cfg(law, dt, nsteps, k, G, eps, q=q, types=types, kq=kq, ntypes=ntypes,
+                   keep_bytes=keep_bytes)
     else:
-        cfg = _Cfg(law, dt, nsteps, k, G, eps)
+        cfg = _Cfg(law, dt, nsteps, k, G, eps, keep_bytes=keep_bytes)
         sig_t = eps_t = torch.zeros(0, device=x0.device)
     return NBodyLeapfrog.apply(x0, v0, m, sig_t, eps_t, cfg)
