@@ -67,7 +67,11 @@ int vjp_table(int law) {
 // streamed triangle kernel where its slots fit. Sets *planned and the scratch layout.
 // Per Hermite step, gravity and LJC reverse step (us), direct / streamed: 10.8, 11.8,
 // 22.8 / - at 2432, 14.3, 15.6, 26.4 / 16.0, 15.0, 26.0 at 2500, 17.9, 19.5, 36.9 at
-// 3500 against 21.8, 21.4, 37.1 at 4096.
+// 3500 against 21.8, 21.4, 37.1 at 4096. Gravity's jerk and VJP go back to the block-pair
+// tiles at 131072: there the streamed rows leave twice the tiles' slots (jerk 2.7 against
+// 1.4 GB at 131072, 10.8 against 5.4 at 262144; VJP half of that) for 1 to 2% of the time
+// (ms, streamed / tile: jerk 5.51 / 5.58 at 98304, 9.74 / 9.91 at 131072, 38.8 / 39.1 at
+// 262144; VJP 5.70 / 5.82, 10.09 / 10.29, 40.2 / 40.8). The LJC VJP's slots are the tile's.
 int vjp_untiled(int law, int n, int sms, cudaStream_t s, VjpScratch *sc, size_t extra,
                 bool *planned) {
   const bool lj = law == NBODY_LAW_LJC || law == NBODY_LAW_LJC_LINEAR;
@@ -75,7 +79,7 @@ int vjp_untiled(int law, int n, int sms, cudaStream_t s, VjpScratch *sc, size_t 
   *planned = false;
   int slots = 1;
   if (n > 16 * sms) {
-    if (n > 0x7fffffff - 64 * 64) return NBODY_OK;
+    if (n > 0x7fffffff - 64 * 64 || (!lj && n >= 131072)) return NBODY_OK;
     sc->tri = tri_vjp(sc->table, n);
     sc->geom = tri_geom(n, sc->tri->h, sms * sc->tri->per_sm);
     slots = sc->geom.nb + tri_max_row_shares(sc->geom);
