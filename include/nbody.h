@@ -416,6 +416,9 @@ int nbody_set_tuned(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit);
  * (subsets, nbody_forces_static, a j-split of the caller's, sizes whose partial sums
  * would pass the limit) take the stored tile. */
 int nbody_set_stored(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit);
+/* Whether (law, n-bucket) has an entry: 0 none, 1 a stored one, 2 an installed one
+ * (nbody_set_tuned, nbody_tune); -1 for a bad argument. */
+int nbody_tuned_kind(int32_t law, int32_t log2n);
 /* Query the tile-table entry of (law, n): the installed or stored one, else the
  * table's default row. */
 int nbody_get_config(int32_t law, int64_t n, int32_t *tile, int32_t *jsplit);
@@ -435,9 +438,9 @@ int nbody_workspace_size(const nbody_params *params, int64_t n, int32_t report_r
  * configurations instead). Every tile x j-split in {0 (auto), 1, 2, 4, 8, 16,
  * 32} that fits n (Newton-symmetric tiles: the splits their plan takes, and only
  * where their partial-sum cap admits n) is run once to warm up and `reps` (1..1000) more times, timed
- * with CUDA events on `stream`; the median decides. The fastest is installed
- * with nbody_set_tuned for bucket floor(log2 n) (with nbody_set_stored where the
- * library's streamed kernel is faster still) and returned in best_tile,
+ * with CUDA events on `stream`; the median decides. The fastest becomes the entry of
+ * bucket floor(log2 n) (nbody_set_stored; where a default call would run a direct or
+ * streamed kernel and the tile is faster, nbody_set_tuned) and is returned in best_tile,
  * best_jsplit and best_ms (milliseconds per call; any may be NULL). What is
  * timed: tables 0-2 nbody_forces (law = table), 4 nbody_forces with
  * NBODY_FIXED_POINT (eps2 > 0), 5 / 6 / 8 nbody_adjoint (gravity / LJC / LJC

@@ -43,7 +43,7 @@ EXPORTS = (
     "nbody_pack_grav", "nbody_pack_ljc", "nbody_forces", "nbody_step",
     "nbody_batch_plan_create", "nbody_batch_plan_destroy", "nbody_batch_plan_particles",
     "nbody_batch_run", "nbody_forces_batched", "nbody_adjoint", "nbody_adjoint_leapfrog",
-    "nbody_tile_count", "nbody_tile_info", "nbody_set_tuned", "nbody_set_stored",
+    "nbody_tile_count", "nbody_tile_info", "nbody_set_tuned", "nbody_set_stored", "nbody_tuned_kind",
     "nbody_get_config",
     "nbody_timing_enable", "nbody_timing_read", "nbody_peak_probe", "nbody_forces_static",
     "nbody_forces_subset", "nbody_forces_jerk", "nbody_hermite_step", "nbody_selftest_timeout",
@@ -120,6 +120,7 @@ def load(path: str | None = None):
                                 ctypes.c_int),
             "nbody_set_tuned": ([i32, i32, i32, i32], ctypes.c_int),
             "nbody_set_stored": ([i32, i32, i32, i32], ctypes.c_int),
+            "nbody_tuned_kind": ([i32, i32], ctypes.c_int),
             "nbody_timing_enable": ([i32], ctypes.c_int),
             "nbody_peak_probe": ([i32, i32, ctypes.POINTER(f64), ctypes.POINTER(f64)],
                                  ctypes.c_int),

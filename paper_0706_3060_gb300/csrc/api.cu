@@ -610,6 +610,15 @@ int nbody_set_stored(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit) {
   return set_tuned(law, log2n, tile, jsplit, false);
 }
 
+int nbody_tuned_kind(int32_t law, int32_t log2n) {
+  clear_error();
+  if (law < 0 || law >= kTables || log2n < 0 || log2n >= 64) return -1;
+  int tile = -1, jsplit = 0;
+  bool by_caller = false;
+  tuned_entry(law, log2n, &tile, &jsplit, &by_caller);
+  return tile < 0 ? 0 : by_caller ? 2 : 1;
+}
+
 int nbody_get_config(int32_t law, int64_t n, int32_t *tile, int32_t *jsplit) {
   clear_error();
   if (law < 0 || law >= kTables) return set_error_msg(NBODY_EINVAL, "bad law %d", law);

@@ -64,7 +64,7 @@ int vjp_table(int law) {
 
 // A default call's kernel without a tile: up to one wave of direct CTAs (two of 8 targets
 // on every SM; 2432 particles on 152) a direct launch (direct_kernel.cuh), above the
-// streamed triangle kernel where its slots fit. Sets *planned and the scratch layout.
+// streamed triangle kernel where its slots fit; false where a tile runs.
 // Per Hermite step, gravity and LJC reverse step (us), direct / streamed: 10.8, 11.8,
 // 22.8 / - at 2432, 14.3, 15.6, 26.4 / 16.0, 15.0, 26.0 at 2500, 17.9, 19.5, 36.9 at
 // 3500 against 21.8, 21.4, 37.1 at 4096. Gravity's jerk and VJP go back to the block-pair
@@ -72,22 +72,30 @@ int vjp_table(int law) {
 // 1.4 GB at 131072, 10.8 against 5.4 at 262144; VJP half of that) for 1 to 2% of the time
 // (ms, streamed / tile: jerk 5.51 / 5.58 at 98304, 9.74 / 9.91 at 131072, 38.8 / 39.1 at
 // 262144; VJP 5.70 / 5.82, 10.09 / 10.29, 40.2 / 40.8). The LJC VJP's slots are the tile's.
-int vjp_untiled(int law, int n, int sms, cudaStream_t s, VjpScratch *sc, size_t extra,
-                bool *planned) {
-  const bool lj = law == NBODY_LAW_LJC || law == NBODY_LAW_LJC_LINEAR;
-  const int blocks = (lj || law == kLawGAJ) ? 2 : 1;
-  *planned = false;
-  int slots = 1;
-  if (n > 16 * sms) {
-    if (n > 0x7fffffff - 64 * 64 || (!lj && n >= 131072)) return NBODY_OK;
-    sc->tri = tri_vjp(sc->table, n);
-    sc->geom = tri_geom(n, sc->tri->h, sms * sc->tri->per_sm);
-    slots = sc->geom.nb + tri_max_row_shares(sc->geom);
-    if (double(blocks) * slots * n * sizeof(float4) > sym_part_cap()) {
-      sc->tri = nullptr;
-      return NBODY_OK;
-    }
-  }
+struct VjpUntiled {
+  const TriDesc *tri;  // null: a direct launch
+  TriGeom geom;
+  int slots;
+  int blocks;          // float4 rows of a particle's sums
+};
+bool vjp_untiled_plan(int table, int64_t n, int sms, VjpUntiled *u) {
+  const bool lj = table == kTableVjpLJC || table == kTableVjpLJCLin;
+  u->blocks = (lj || table == kTableJerk) ? 2 : 1;
+  u->tri = nullptr;
+  u->slots = 1;
+  if (n <= 16 * sms) return true;
+  if (n > 0x7fffffff - 64 * 64 || (!lj && n >= 131072)) return false;
+  u->tri = tri_vjp(table, n);
+  u->geom = tri_geom(int(n), u->tri->h, sms * u->tri->per_sm);
+  u->slots = u->geom.nb + tri_max_row_shares(u->geom);
+  return double(u->blocks) * u->slots * double(n) * sizeof(float4) <= sym_part_cap();
+}
+
+// Its scratch layout.
+int vjp_untiled(const VjpUntiled &u, int n, cudaStream_t s, VjpScratch *sc, size_t extra) {
+  sc->tri = u.tri;
+  sc->geom = u.geom;
+  const int blocks = u.blocks, slots = u.slots;
   const size_t part = round_up(size_t(blocks) * slots * size_t(n) * sizeof(float4), 256);
   const size_t lo = sc->tri ? 0 : part;
   const int per_block = sc->tri ? kSlotParts : 256;
@@ -109,7 +117,6 @@ int vjp_untiled(int law, int n, int sms, cudaStream_t s, VjpScratch *sc, size_t 
   sc->bstride = (long long)slots * n;
   sc->d = nullptr;
   sc->sym_split = 1;
-  *planned = true;
   return NBODY_OK;
 }
 
@@ -165,9 +172,8 @@ int vjp_prepare(int law, int n, int tile, int jsplit, int sms, cudaStream_t s, V
   sc->table = table;
   sc->tri = nullptr;
   if (tile < 0 && jsplit <= 0 && atomic_mode < 2 && !tuned_by_caller(table, n)) {
-    bool planned = false;
-    NB_TRY(vjp_untiled(law, n, sms, s, sc, extra, &planned));
-    if (planned) return NBODY_OK;
+    VjpUntiled u{};
+    if (vjp_untiled_plan(table, n, sms, &u)) return vjp_untiled(u, n, s, sc, extra);
   }
   int count = 0;
   const VjpDesc *tiles = vjp_tiles(table, &count);
@@ -521,6 +527,11 @@ int check_jerk_params(const nbody_params *params, uint32_t extra_flags) {
 }
 
 }  // namespace
+
+bool nbody::vjp_runs_untiled(int table, int64_t n, int sms) {
+  VjpUntiled u{};
+  return vjp_untiled_plan(table, n, sms, &u);
+}
 
 extern "C" {
 

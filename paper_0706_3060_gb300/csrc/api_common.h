@@ -205,6 +205,9 @@ size_t round_up(size_t x, size_t a);
 // preferred to the streamed kernels; otherwise a stored entry.
 int set_tuned(int law, int log2n, int tile, int jsplit, bool by_caller);
 bool tuned_by_caller(int law, int64_t n);
+// Whether calls of a VJP or jerk table that leave the configuration to the library run a
+// kernel without a tile at n particles (unless an entry was installed by the caller).
+bool vjp_runs_untiled(int table, int64_t n, int sms);
 void tuned_entry(int law, int log2n, int *tile, int *jsplit, bool *by_caller);
 int get_config(int law, int64_t n, int *tile, int *jsplit);
 const char *last_error_text();

@@ -52,6 +52,17 @@ int run_once(int table, const void *pos, const void *prm, int64_t n, float eps2,
   }
 }
 
+// Whether the call with tile == -1 runs a kernel without a tile (direct or streamed) where
+// no entry was installed by the caller.
+bool default_untiled(int table, int64_t n, float eps2, int sms) {
+  if (table == kTableGravFixed) return false;
+  if (table >= kTableVjpGrav) return vjp_runs_untiled(table, n, sms);
+  Plan1 plan{};
+  return plan_single(table, n, -1, 0, sms, &plan, true,
+                     table == NBODY_LAW_GRAV && eps2 > 0.0f) == NBODY_OK &&
+         (plan.direct || plan.tri);
+}
+
 // Median time of `reps` runs of call(), each between two events on `s`.
 template <class F>
 int time_call(int reps, std::vector<float> &ts, float *median, cudaStream_t s, F &&call) {
@@ -164,20 +175,22 @@ int nbody_tune(int32_t table, const void *pos_m, const void *prm, int64_t n, flo
   if (bt < 0) return set_error_msg(NBODY_EINVAL, "no tile fits n = %lld", (long long)n);
   int lg = 0;
   while ((int64_t(1) << (lg + 1)) <= n && lg < 62) ++lg;
-  // Install the winner; where the streamed kernel that a default call would run is
-  // faster still, as a stored entry, which leaves such calls with it.
+  // Store the winner, which leaves default calls with the direct or streamed kernel that
+  // they run; installed, before that kernel, only where there is one and the tile is faster.
   int old_tile = -1, old_js = 0;
   bool old_caller = false;
   tuned_entry(table, lg, &old_tile, &old_js, &old_caller);
   NB_TRY(set_tuned(table, lg, bt, bj, false));
-  st = run_once(table, pos_m, prm, n, eps2, -1, 0, o0, o1, om, s);
   float lib_ms = -1.0f;
-  if (st == NBODY_OK) st = time_call(reps, ts, &lib_ms, s, [&]() {
-    return run_once(table, pos_m, prm, n, eps2, -1, 0, o0, o1, om, s);
-  });
-  if (st != NBODY_OK) {
-    set_tuned(table, lg, old_tile, old_js, old_caller);
-    return st;
+  if (default_untiled(table, n, eps2, sms)) {
+    st = run_once(table, pos_m, prm, n, eps2, -1, 0, o0, o1, om, s);
+    if (st == NBODY_OK) st = time_call(reps, ts, &lib_ms, s, [&]() {
+      return run_once(table, pos_m, prm, n, eps2, -1, 0, o0, o1, om, s);
+    });
+    if (st != NBODY_OK) {
+      set_tuned(table, lg, old_tile, old_js, old_caller);
+      return st;
+    }
   }
   if (lib_ms > best) NB_TRY(set_tuned(table, lg, bt, bj, true));
   if (best_tile) *best_tile = bt;
