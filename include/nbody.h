@@ -85,7 +85,16 @@ enum {
                                         with compensation); Newton-symmetric
                                         tiles always sum within a block pair
                                         plainly, and with this flag also add
-                                        their per-block partials plainly      */
+                                        their per-block partials plainly. The
+                                        direct and streamed kernels of default
+                                        calls (tile -1, jsplit 0) add 16 to 128
+                                        sources at a time plainly and such sums
+                                        with compensation; there the flag only
+                                        makes nbody_forces, nbody_step and batch
+                                        plans on the streamed kernels add their
+                                        partials plainly: one direct launch,
+                                        jerk, Hermite steps and VJPs give the
+                                        same bits with and without it          */
     NBODY_ACC_VALID = 1u << 3,       /* nbody_step: acc already holds a(x) for
                                         the entry positions                    */
     NBODY_ACCUMULATE = 1u << 4,      /* nbody_adjoint: add into the outputs    */
@@ -311,8 +320,10 @@ typedef struct {
 typedef struct nbody_batch_plan nbody_batch_plan;
 
 /* Build the work list (longest items first) for a host table of systems.
- * flags: NBODY_PRECISE_RSQRT / NBODY_NO_COMPENSATION. tile = -1 picks the
- * tuned configuration. Allocates device memory; no stream work. */
+ * flags: NBODY_PRECISE_RSQRT / NBODY_NO_COMPENSATION. tile = -1 runs the streamed
+ * kernel; where nbody_set_tuned installed an entry of table 3, or its partial sums
+ * would pass the limit (an eighth of the device's memory, at most 16 GiB), the
+ * table's entry or default row. Allocates device memory; no stream work. */
 int nbody_batch_plan_create(const nbody_system *systems, int32_t nsys, uint32_t flags,
                             int32_t tile, nbody_batch_plan **plan);
 int nbody_batch_plan_destroy(nbody_batch_plan *plan);
@@ -410,11 +421,14 @@ int nbody_tile_info(int32_t law, int32_t tile, int32_t *threads, int32_t *i_per_
  * tile -1 removes the entry. */
 int nbody_set_tuned(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit);
 /* The same for an entry of a stored table, which does not stand in the way of the
- * streamed kernels: calls with tile == -1 and jsplit == 0 for which the library has
- * one (nbody_forces and nbody_step without NBODY_FIXED_POINT) run that unless
- * nbody_set_tuned or nbody_tune installed an entry for the size; the other calls
- * (subsets, nbody_forces_static, a j-split of the caller's, sizes whose partial sums
- * would pass the limit) take the stored tile. */
+ * direct and streamed kernels. Calls with tile == -1 and jsplit == 0 run those where the
+ * library has one -- nbody_forces, nbody_step, nbody_forces_subset, the jerk and Hermite
+ * calls, the adjoint calls and batch plans, without NBODY_FIXED_POINT -- unless
+ * nbody_set_tuned or nbody_tune installed an entry for the size. The other calls
+ * (nbody_forces_static, a j-split of the caller's, larger systems: gravity forces from
+ * 114688 particles, 163840 without softening or with plain sums, gravity's jerk and VJP
+ * from 131072, subsets of more than two million sources, partial sums beyond the limit)
+ * take the stored tile. */
 int nbody_set_stored(int32_t law, int32_t log2n, int32_t tile, int32_t jsplit);
 /* Whether (law, n-bucket) has an entry: 0 none, 1 a stored one, 2 an installed one
  * (nbody_set_tuned, nbody_tune); -1 for a bad argument. */
