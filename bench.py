@@ -550,9 +550,9 @@ def roofline_by_form(nb, torch, dev):
         out[name] = {"n": n, "ops_per_pair": ops, "kernel_ms": ms,
                      "gpairs_per_s": pairs / (ms * 1e-3) / 1e9, "achieved_tflops": t,
                      "frac": t / peak}
-    # the batched persistent kernel over the 512-system ensemble: one-sided tiles do
-    # 12 ops per gravity pair and 23 per LJC pair; the Newton-symmetric tiles 16 and
-    # 26 per unordered pair
+    # the batched kernels over the 512-system ensemble: the streamed kernel, which default
+    # plans run, and the Newton-symmetric tiles do 16 ops per unordered gravity pair and 26
+    # per LJC pair, one-sided tiles 12 and 23 per ordered pair
     ens = workloads.ensemble(nsys=512, seed=3)
     bpos, bvel, bprm, table = _ensemble_arrays(nb, torch, dev, ens)
     bacc = torch.zeros_like(bpos)
@@ -561,14 +561,14 @@ def roofline_by_form(nb, torch, dev):
     pgu = sum(x.n * (x.n - 1) / 2 for x in ens.systems if isinstance(x, workloads.GravInput))
     plu = sum(x.n * (x.n - 1) / 2 for x in ens.systems if not isinstance(x, workloads.GravInput))
     btile, _ = nb.get_config(nb.TABLE_BATCHED, 0)
-    forms = [("batched ensemble (one-sided)", 9)]
+    forms = [("batched ensemble (streamed, default)", -1), ("batched ensemble (one-sided)", 9)]
     if nb.tile_info(nb.TABLE_BATCHED, btile)["symmetric"]:
-        forms.insert(0, ("batched ensemble (Newton-symmetric)", btile))
+        forms.insert(1, ("batched ensemble (Newton-symmetric tile)", btile))
     for name, tl in forms:
         plan = nb.BatchPlan(table, tile=tl)
         ms = kernel_ms(lambda: plan.run(bpos, bvel, bacc, bprm, nsteps=0, graph=False), 0)
         plan.close()
-        if nb.tile_info(nb.TABLE_BATCHED, tl)["symmetric"]:
+        if tl < 0 or nb.tile_info(nb.TABLE_BATCHED, tl)["symmetric"]:
             ops = SYM_OPS_PER_UNORDERED_PAIR * pgu + SYM_LJC_OPS_PER_UNORDERED_PAIR * plu
         else:
             ops = 12 * pg2 + 23 * pl2
