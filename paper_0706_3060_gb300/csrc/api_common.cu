@@ -379,11 +379,8 @@ int launch_direct(const DirectArgs &a, const DirectPlan &plan, uint32_t flags, b
                                                      : direct_ljclin;
   DirectArgs d = a;
   d.slices = plan.slices;
-  // 16 targets' gravity with potentials leave one CTA on an SM: 8 (the same sums: their
-  // order depends on the slices alone)
-  const bool big = plan.big && !(a.law == NBODY_LAW_GRAV && pot);
   const TimerMark tm = timed ? timer_begin(0, s) : TimerMark{};
-  const cudaError_t e = go(d, big, pot, (flags & NBODY_PRECISE_RSQRT) != 0, s);
+  const cudaError_t e = go(d, plan.big, pot, (flags & NBODY_PRECISE_RSQRT) != 0, s);
   timer_end(tm, s);
   if (e != cudaSuccess)
     return set_error_msg(e == cudaErrorNoKernelImageForDevice ? NBODY_EUNSUPPORTED : NBODY_ECUDA,

@@ -9,7 +9,7 @@ using Law = TriGrav<POT, PRECISE, true>;
 }
 
 cudaError_t direct_grav(const DirectArgs &a, bool big, bool pot, bool precise, cudaStream_t s) {
-  return direct_law<Law, 4>(a, big, pot, precise, s);
+  return direct_law<Law, 4, false>(a, big, pot, precise, s);
 }
 
 }  // namespace nbody

@@ -49,20 +49,23 @@ inline cudaError_t direct_go(const DirectArgs &a, cudaStream_t s) {
 
 // U: sources on their way per thread (the L2 latency of about 700 cycles against the
 // time of one source; 16 targets of gravity with 1 / 2 / 4: 61 / 86 / 49 us for 1500
-// targets of 65536).
-template <template <bool, bool> class LAW, int U>
+// targets of 65536). Without BIG_POT potentials take 8 targets (16 would leave one CTA on an SM;
+// the same sums: their order depends on the slices alone).
+template <template <bool, bool> class LAW, int U, bool BIG_POT>
 inline cudaError_t direct_law(const DirectArgs &a, bool big, bool pot, bool precise,
                               cudaStream_t s) {
-  if (big) {
-    if (pot)
-      return precise ? direct_go<LAW<true, true>, 8, U>(a, s)
-                     : direct_go<LAW<true, false>, 8, U>(a, s);
-    return precise ? direct_go<LAW<false, true>, 8, U>(a, s)
-                   : direct_go<LAW<false, false>, 8, U>(a, s);
-  }
-  if (pot)
+  if (pot) {
+    if constexpr (BIG_POT) {
+      if (big)
+        return precise ? direct_go<LAW<true, true>, 8, U>(a, s)
+                       : direct_go<LAW<true, false>, 8, U>(a, s);
+    }
     return precise ? direct_go<LAW<true, true>, 4, U>(a, s)
                    : direct_go<LAW<true, false>, 4, U>(a, s);
+  }
+  if (big)
+    return precise ? direct_go<LAW<false, true>, 8, U>(a, s)
+                   : direct_go<LAW<false, false>, 8, U>(a, s);
   return precise ? direct_go<LAW<false, true>, 4, U>(a, s)
                  : direct_go<LAW<false, false>, 4, U>(a, s);
 }

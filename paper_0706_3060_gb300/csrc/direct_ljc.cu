@@ -9,7 +9,7 @@ using Law = TriLjc<false, POT, PRECISE>;
 }
 
 cudaError_t direct_ljc(const DirectArgs &a, bool big, bool pot, bool precise, cudaStream_t s) {
-  return direct_law<Law, 2>(a, big, pot, precise, s);
+  return direct_law<Law, 2, true>(a, big, pot, precise, s);
 }
 
 }  // namespace nbody

@@ -9,7 +9,7 @@ using Law = TriLjc<true, POT, PRECISE>;
 }
 
 cudaError_t direct_ljclin(const DirectArgs &a, bool big, bool pot, bool precise, cudaStream_t s) {
-  return direct_law<Law, 2>(a, big, pot, precise, s);
+  return direct_law<Law, 2, true>(a, big, pot, precise, s);
 }
 
 }  // namespace nbody
