@@ -14,19 +14,19 @@
 // steps, eight per warp, and the four parts of their source-side sums added in
 // shared memory.
 //
-// Why this shape. The packed FP32 unit bounds the loop (an f32x2 instruction holds its
-// issue port for two cycles, one whose three operands share a register bank for longer;
-// each MUFU adds 1.3 cycles: about 39 of the 32 cycles that 16 operations on 64 targets
-// need), and per source-step a lane spends about 25 instructions besides the pairs:
-// 2 H targets per step share them. Pairs of targets instead of pairs of sources in the
+// Why this shape. The packed FP32 unit bounds the loop: an f32x2 instruction holds its
+// issue port for two cycles, so that the 16 operations of one register group (64 targets of
+// a warp) take 32 at least; they take about 39, because one whose three operands share a
+// register bank holds it longer and each MUFU adds 1.3. Per source-step a lane spends about
+// 25 instructions besides the pairs: 2 H targets per step share them. Pairs of targets instead of pairs of sources in the
 // f32x2 halves halve the registers per target (no duplicated target words), so a lane
 // holds up to 16 targets at 8 warps per SM. Equal shares leave no partial wave: all CTAs
 // are resident from the start (taken from a queue in smaller pieces instead, 3 to 6%
 // more: 82 us against 77.5 at 16384, 298 against 287 at 32768). Two CTAs of four warps
 // per SM: one of eight, whose warps keep step with each other, took 5% longer.
-// Leapfrog steps inside a call (us), block-pair tile -> here: gravity 36.4 -> 27.5 at
-// 8192, 91.8 -> 80.1 at 16384, 308 -> 294 at 32768; LJC 44.9 -> 36.2, 129.6 -> 116.9,
-// 475 -> 441, and 1831 -> 1721 at 65536 (80% of the FP32 lane peak).
+// Leapfrog steps inside a call (us), block-pair tile -> here: gravity 36.4 -> 28.4 at
+// 8192, 91.8 -> 80.7 at 16384, 308 -> 295 at 32768; LJC 44.9 -> 36.5, 129.6 -> 117.2,
+// 475 -> 440, and 1831 -> 1721 at 65536 (80% of the FP32 lane peak).
 //
 // Sums. A target's sum is plain FP32 over the sources that one warp meets in kChunk groups
 // (128 with 16 groups, and the left-over ones), then over at most four such sums (a

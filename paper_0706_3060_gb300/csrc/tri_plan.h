@@ -8,9 +8,9 @@
 // source group g >= 2 h b: the first 2 h groups of a row are its own particles, the
 // others lie beyond it. The units are put in a line, row after row, each of cost 1; a
 // row costs kTriRowCost more, for loading its targets and adding up its sums. Within a
-// row the own units, which mask what they do not count, are spread evenly among the
-// others (tri_own), so that every share of a row gets its part of them. The line is cut
-// into nshare shares of equal cost.
+// row the own units, whose pairs are met twice but from one side (tri_kernel.cuh), are
+// spread evenly among the others (tri_own), so that every share of a row gets its part of
+// them. The line is cut into nshare shares of equal cost.
 #pragma once
 
 #include <cstdint>
