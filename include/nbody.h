@@ -135,7 +135,9 @@ int nbody_version(void);
 /* Thread-local message for the last non-OK status returned on this thread. */
 const char *nbody_last_error(void);
 
-/* Release the library's internal workspaces on the current device.
+/* Release the library's internal workspaces on the current device, those among them that
+ * graphs captured from calls of this library use (destroy such graphs first; until then
+ * a workspace that a captured call used is kept when a later call needs a larger one).
  * Synchronizes the device. */
 int nbody_release(void);
 

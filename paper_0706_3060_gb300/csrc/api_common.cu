@@ -25,9 +25,13 @@ thread_local std::string t_err;
 struct Arena {
   void *ptr = nullptr;
   size_t cap = 0;
+  bool captured = false;  // handed to a call under stream capture: a graph holds its address
 };
 
 std::mutex g_mu;
+// Outgrown arenas that graphs hold, until release_all. A stream's arenas grow by a quarter
+// at least, so that those of captured calls take at most four times the newest.
+std::vector<void *> g_held;
 std::map<std::pair<int, cudaStream_t>, Arena> g_ws;
 std::map<std::pair<int, cudaStream_t>, Arena> g_stage;
 std::map<int, int *> g_err_word;  // device -> address of g_dev_err_word there
@@ -46,9 +50,10 @@ int grow(std::map<std::pair<int, cudaStream_t>, Arena> &tab, cudaStream_t s, siz
   NB_CUDA(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_mu);
   Arena &a = tab[{dev, s}];
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (a.cap < bytes || !a.captured) NB_CUDA(cudaStreamIsCapturing(s, &cs));
+  if (cs != cudaStreamCaptureStatusNone && a.cap >= bytes) a.captured = true;
   if (a.cap < bytes) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    NB_CUDA(cudaStreamIsCapturing(s, &cs));
     if (cs != cudaStreamCaptureStatusNone)
       return set_error_msg(NBODY_EINVAL,
                            "workspace of %zu bytes needed during stream capture; run the "
@@ -56,9 +61,11 @@ int grow(std::map<std::pair<int, cudaStream_t>, Arena> &tab, cudaStream_t s, siz
                            bytes);
     // The old buffer may still be in use by work queued on this stream: free it
     // in stream order, then allocate the larger one.
-    if (a.ptr) NB_CUDA(cudaFreeAsync(a.ptr, s));
-    a.ptr = nullptr;
-    a.cap = 0;
+    if (a.ptr && a.captured)
+      g_held.push_back(a.ptr);
+    else if (a.ptr)
+      NB_CUDA(cudaFreeAsync(a.ptr, s));
+    a = Arena{};
     size_t want = bytes + bytes / 4 + 4096;
     cudaError_t e = cudaMallocAsync(&a.ptr, want, s);
     if (e != cudaSuccess) {
@@ -182,6 +189,8 @@ void release_all() {
       if (kv.second.ptr) cudaFree(kv.second.ptr);
     tab->clear();
   }
+  for (void *q : g_held) cudaFree(q);
+  g_held.clear();
 }
 
 namespace {
