@@ -11,14 +11,16 @@
 // so results are bitwise reproducible.
 //
 // Sums. A thread adds 32 sources in plain FP32, then such sums in shared memory, and the
-// first two exchanges between lanes are plain. Gravity's forces (kFine) fold every 16
-// sources (none up to 20), add the folds with TwoSum and, above 2048 particles, compensate
-// every exchange: a close pair's large pull is rounded again with each later add. Rms errors
-// against 64 bits, plain / so / tile: 1500 targets of 65536 3.75e-8 / 3.60e-8 / 3.60e-8,
-// 4000 of 131072 3.66e-8 / 3.50e-8 / 3.49e-8, all of 3300 5.03e-8 / 4.93e-8 / 5.07e-8.
-// Time (us, calls in a loop), plain / so: 58.6 / 62.5, 253 / 269, and a step of 4001
-// particles 12.7 / 12.4. The LJC laws' errors are those of their pair terms (1.2e-6 either
-// way), and the VJPs and the jerk run here up to 2432 particles, without folds.
+// first two exchanges between lanes are plain. Gravity's forces (kFine) fold every 12
+// sources (none up to 20), add the folds with compensation and, above 2048 particles,
+// compensate every exchange: a close pair's large pull is rounded again with each later add.
+// Rms errors against 64 bits, plain / so / tile: 1500 targets of 65536 3.80e-8 / 3.66e-8 /
+// 3.65e-8, 4000 of 131072 3.66e-8 / 3.46e-8 / 3.49e-8, the same with a close companion for
+// every particle 1.55e-7 / 1.35e-7 / 1.35e-7, all of 3300 5.03e-8 / 4.93e-8 / 5.07e-8. Time
+// (us, calls in a loop), plain / so: 58.6 / 64.5, 253 / 277, and a step of 4001 particles
+// 12.7 / 12.4; folds of 16 4% less and errors up to 1% above the tiles'. The LJC laws'
+// errors are those of their pair terms (1.2e-6 either way), and the VJPs and the jerk run
+// here up to 2432 particles, without folds.
 //
 // What bounds it: launch and latency up to about 1500 particles (one launch where the
 // tile path takes an interleave, a force and a finalize launch), then the packed FP32
@@ -43,9 +45,17 @@ constexpr int kDirectWarps = kDirectThreads / 32;
 constexpr int kDirectFold = 32;  // sources per register sum
 // Laws with finer sums (kFine): sources per register sum, the most that are added without
 // folds, and particles up to which the first two exchanges between lanes are plain
-constexpr int kFineFold = 16, kFineChain = 20, kFineFew = 2048;
+constexpr int kFineFold = 12, kFineChain = 20, kFineFew = 2048;
 template <class L>
 constexpr int direct_chain() { return L::kFine ? kFineChain : kDirectFold; }
+
+// Adds a into the sum h with low part l: three operations of TwoSum's six, exact where h is
+// the larger one; where a is (a close pair's pull arrives), rounded once more.
+__device__ __forceinline__ void fold_add(float &h, float &l, float a) {
+  const float s = __fadd_rn(h, a);
+  l = __fadd_rn(l, __fsub_rn(a, __fsub_rn(s, h)));
+  h = s;
+}
 
 struct DirectArgs {
   const float4 *pos;  // sources (x, y, z, m)
@@ -131,28 +141,30 @@ __global__ void __launch_bounds__(kDirectThreads,
 #pragma unroll
   for (int u = 0; u < U; ++u)
     L::load(a.pos, a.prm, a.vec, min(b0 + u, b1) * kDirectThreads + tid, a.n, P[u]);
+  int fold_at = b0;  // the block after the last fold
   for (int b = b0; b < b1; b += U) {
     // every kFold sources the sums go to this thread's own words in shared memory:
     // a close pair's large pull is not rounded again with each of hundreds of sources
-    if (many && b > b0 && ((b - b0) & (kFold - 1)) == 0) {
+    if (many && b - fold_at == kFold) {
+      const bool first = fold_at == b0;
+      fold_at = b;
 #pragma unroll
       for (int r = 0; r < H; ++r)
 #pragma unroll
         for (int c = 0; c < NS; ++c) {
-          float2 *f = folded + (r * NS + c) * kDirectThreads + tid;
+          const int at = (r * NS + c) * kDirectThreads + tid;
           if constexpr (L::kFine) {
-            float2 *e = f + H * NS * kDirectThreads;
-            float2 h = A[r][c], l = make_float2(0.0f, 0.0f);
-            if (b > b0 + kFold) {
-              h = *f;
-              l = *e;
-              comp_add(h.x, l.x, A[r][c].x);
-              comp_add(h.y, l.y, A[r][c].y);
+            float4 *f = reinterpret_cast<float4 *>(folded) + at;  // sums, then low parts
+            float4 t = make_float4(A[r][c].x, A[r][c].y, 0.0f, 0.0f);
+            if (!first) {
+              t = *f;
+              fold_add(t.x, t.z, A[r][c].x);
+              fold_add(t.y, t.w, A[r][c].y);
             }
-            *f = h;
-            *e = l;
+            *f = t;
           } else {
-            *f = b > b0 + kFold ? __fadd2_rn(*f, A[r][c]) : A[r][c];
+            float2 *f = folded + at;
+            *f = first ? A[r][c] : __fadd2_rn(*f, A[r][c]);
           }
           A[r][c] = make_float2(0.0f, 0.0f);
         }
@@ -180,14 +192,14 @@ __global__ void __launch_bounds__(kDirectThreads,
     for (int r = 0; r < H; ++r)
 #pragma unroll
       for (int c = 0; c < NS; ++c) {
-        const float2 *f = folded + (r * NS + c) * kDirectThreads + tid;
+        const int at = (r * NS + c) * kDirectThreads + tid;
         if constexpr (L::kFine) {
-          float2 h = *f, l = f[H * NS * kDirectThreads];
-          comp_add(h.x, l.x, A[r][c].x);
-          comp_add(h.y, l.y, A[r][c].y);
-          A[r][c] = __fadd2_rn(h, l);
+          float4 t = reinterpret_cast<const float4 *>(folded)[at];
+          fold_add(t.x, t.z, A[r][c].x);
+          fold_add(t.y, t.w, A[r][c].y);
+          A[r][c] = make_float2(t.x + t.z, t.y + t.w);
         } else {
-          A[r][c] = __fadd2_rn(*f, A[r][c]);
+          A[r][c] = __fadd2_rn(folded[at], A[r][c]);
         }
       }
   }
