@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kDirectThreads,
         g = 0;
       }
     }
-    L::load(a.pos, a.prm, a.vec, g >= 0 ? g : a.n, a.n, w);
+    L::template load<true>(a.pos, a.prm, a.vec, g >= 0 ? g : a.n, a.n, w);
     L::as_target(w);
 #pragma unroll
     for (int c = 0; c < L::kWords; ++c) words[c][tid] = w[c];
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kDirectThreads,
   float P[U][L::kWords];
 #pragma unroll
   for (int u = 0; u < U; ++u)
-    L::load(a.pos, a.prm, a.vec, min(b0 + u, b1) * kDirectThreads + tid, a.n, P[u]);
+    L::template load<true>(a.pos, a.prm, a.vec, min(b0 + u, b1) * kDirectThreads + tid, a.n, P[u]);
   int fold_at = b0;  // the block after the last fold
   for (int b = b0; b < b1; b += U) {
     // every kFold sources the sums go to this thread's own words in shared memory:
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kDirectThreads,
                                         tidx[2 * r + 1] != j);
       }
       if (b + u + U < b1)
-        L::load(a.pos, a.prm, a.vec, j + U * kDirectThreads, a.n, P[u]);
+        L::template load<true>(a.pos, a.prm, a.vec, j + U * kDirectThreads, a.n, P[u]);
     }
   }
   if (many) {

@@ -13,11 +13,13 @@
 // (Newton's third law), applied when J is stored. kChunk, kParts: lengths of the plain sums;
 // kFine, kLow: compensated sums and the potential's low parts (tri_kernel.cuh, Sums).
 //
-// The particles' words are read with ordinary loads: the finalize in front of these
-// kernels lets them be placed early (griddep_launch) and writes positions, velocities and
+// The streamed kernels read the particles' words with ordinary loads: the finalize in front
+// of them lets them be placed early (griddep_launch) and writes positions, velocities and
 // lambda while they are, and only ordinary loads are ordered by griddep_start; the
-// non-coherent ones (__ldg) want memory that nobody writes as long as the kernel lives.
-// Parameters are written by no kernel of a chain.
+// non-coherent ones (__ldg, NC) want memory that nobody writes as long as the kernel lives.
+// The direct kernels, in front of which nothing triggers early, live only after the last
+// write, and read through that path (steps of 4001 particles 11.6 us, with ordinary loads
+// 12.2). Parameters are written by no kernel of a chain.
 //
 // The source-side sums are plain floats updated with scalar fused multiply-adds: they
 // are added up and handed from lane to lane one word at a time (tri_kernel.cuh), and
@@ -29,6 +31,11 @@
 #include "device_common.cuh"
 
 namespace nbody {
+
+template <bool NC>
+__device__ __forceinline__ float4 load4(const float4 *p) {
+  return NC ? __ldg(p) : *p;
+}
 
 __device__ __forceinline__ float2 bcast(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
@@ -61,9 +68,10 @@ struct TriGrav {
   static constexpr bool kFine = FINE, kLow = FINE && POT;
   static constexpr int kChunk = FINE ? 8 : 16, kParts = FINE ? 2 : 1;
   // words of particle i, or of the massless pad far away
+  template <bool NC = false>
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *, const float4 *,
                                               int i, int n, float (&w)[kWords]) {
-    const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    const float4 p = i < n ? load4<NC>(p0 + i) : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
     w[0] = p.x;
     w[1] = p.y;
     w[2] = p.z;
@@ -114,9 +122,10 @@ struct TriLjc {
   static constexpr unsigned kFlip = 0x7;
   static constexpr bool kFine = false, kLow = false;
   static constexpr int kChunk = 16, kParts = 1;
+  template <bool NC = false>
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *p1, const float4 *,
                                               int i, int n, float (&w)[kWords]) {
-    const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    const float4 p = i < n ? load4<NC>(p0 + i) : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
     const float4 q = i < n ? __ldg(p1 + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     w[0] = p.x;
     w[1] = p.y;

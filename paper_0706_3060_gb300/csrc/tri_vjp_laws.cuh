@@ -9,10 +9,11 @@
 namespace nbody {
 
 // Words x, y, z, m of particle i and three more from its element of `p2`.
+template <bool NC>
 __device__ __forceinline__ void load_pos_and(const float4 *p0, const float4 *p2, int i, int n,
                                              float (&w)[7]) {
-  const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
-  const float4 v = i < n ? p2[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const float4 p = i < n ? load4<NC>(p0 + i) : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+  const float4 v = i < n ? load4<NC>(p2 + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   w[0] = p.x;
   w[1] = p.y;
   w[2] = p.z;
@@ -31,9 +32,10 @@ struct TriJerk {
   static constexpr unsigned kFlip = 0x3f;
   static constexpr bool kFine = false, kLow = false;
   static constexpr int kChunk = 16, kParts = 1;
+  template <bool NC = false>
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *, const float4 *p2,
                                               int i, int n, float (&w)[kWords]) {
-    load_pos_and(p0, p2, i, n, w);
+    load_pos_and<NC>(p0, p2, i, n, w);
   }
   static __device__ __forceinline__ void as_target(float (&w)[kWords]) {
 #pragma unroll
@@ -93,9 +95,10 @@ struct TriGravVjp {
   static constexpr unsigned kFlip = 0xf;
   static constexpr bool kFine = FINE, kLow = false;
   static constexpr int kChunk = FINE ? 4 : 16, kParts = FINE ? 4 : 1;
+  template <bool NC = false>
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *, const float4 *p2,
                                               int i, int n, float (&w)[kWords]) {
-    load_pos_and(p0, p2, i, n, w);
+    load_pos_and<NC>(p0, p2, i, n, w);
   }
   static __device__ __forceinline__ void as_target(float (&w)[kWords]) {
     w[0] = -w[0];
@@ -155,12 +158,13 @@ struct TriLjcVjp {
   static constexpr unsigned kFlip = 0x77;
   static constexpr bool kFine = false, kLow = false;
   static constexpr int kChunk = 16, kParts = 1;
+  template <bool NC = false>
   static __device__ __forceinline__ void load(const float4 *p0, const float4 *p1,
                                               const float4 *p2, int i, int n,
                                               float (&w)[kWords]) {
-    const float4 p = i < n ? p0[i] : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+    const float4 p = i < n ? load4<NC>(p0 + i) : make_float4(1e18f, 1e18f, 1e18f, 0.0f);
     const float4 q = i < n ? __ldg(p1 + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    const float4 l = i < n ? p2[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float4 l = i < n ? load4<NC>(p2 + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     const float inv = i < n ? 1.0f / p.w : 0.0f;
     w[0] = p.x;
     w[1] = p.y;

@@ -34,7 +34,8 @@ def _same(outs):
         assert torch.equal(s, t)
 
 
-@pytest.mark.parametrize("law,n", [("grav", 5001), ("grav", 12289), ("ljc", 2433), ("ljc", 8192)])
+@pytest.mark.parametrize("law,n", [("grav", 1001), ("grav", 4001), ("grav", 5001), ("grav", 12289),
+                                   ("ljc", 777), ("ljc", 2433), ("ljc", 8192)])
 def test_steps(law, n):
     nb = lib()
     pos, vel, prm, kw = _system(law, n)
@@ -48,7 +49,7 @@ def test_steps(law, n):
     _same(outs)
 
 
-@pytest.mark.parametrize("n", [2433, 8191])
+@pytest.mark.parametrize("n", [1001, 2433, 8191])
 def test_hermite(n):
     nb = lib()
     pos, vel, _, kw = _system("grav", n)
@@ -62,7 +63,8 @@ def test_hermite(n):
     _same(outs)
 
 
-@pytest.mark.parametrize("law,n", [("grav", 2433), ("grav", 8191), ("ljc", 2561)])
+@pytest.mark.parametrize("law,n", [("grav", 1001), ("grav", 2433), ("grav", 8191), ("ljc", 777),
+                                   ("ljc", 2561)])
 def test_reverse_sweep(law, n):
     nb = lib()
     pos, vel, prm, kw = _system(law, n)
