@@ -388,6 +388,7 @@ int launch_direct(const DirectArgs &a, const DirectPlan &plan, uint32_t flags, b
                                                      : direct_ljclin;
   DirectArgs d = a;
   d.slices = plan.slices;
+  d.fine = direct_fine(a.idx != nullptr, a.n);
   const TimerMark tm = timed ? timer_begin(0, s) : TimerMark{};
   const cudaError_t e = go(d, plan.big, pot, (flags & NBODY_PRECISE_RSQRT) != 0, s);
   timer_end(tm, s);

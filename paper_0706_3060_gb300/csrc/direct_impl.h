@@ -18,7 +18,7 @@ inline cudaError_t direct_go(const DirectArgs &a, cudaStream_t s) {
   // a thread's folded sums, where its slice has more than one fold
   const int blocks = (a.n + kDirectThreads - 1) / kDirectThreads;
   if ((blocks + a.slices - 1) / a.slices > direct_chain<L>()) {
-    constexpr size_t kBytes = size_t(L::kFine ? 2 : 1) * H * L::kSums * kDirectThreads * sizeof(float2);
+    constexpr size_t kBytes = size_t(H) * L::kSums * kDirectThreads * sizeof(float2);
     cfg.dynamicSmemBytes = kBytes;
     static std::atomic<bool> opted[kMaxDevicesTile];
     int dev = 0;

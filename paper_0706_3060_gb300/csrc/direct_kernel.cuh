@@ -12,13 +12,14 @@
 //
 // Sums. A thread adds 32 sources in plain FP32, then such sums in shared memory, and the
 // first two exchanges between lanes are plain. Gravity's forces (kFine) fold every 12
-// sources (none up to 20), add the folds with compensation and, above 2048 particles,
-// compensate every exchange: a close pair's large pull is rounded again with each later add.
-// Rms errors against 64 bits, plain / so / tile: 1500 targets of 65536 3.80e-8 / 3.66e-8 /
-// 3.65e-8, 4000 of 131072 3.66e-8 / 3.46e-8 / 3.49e-8, the same with a close companion for
-// every particle 1.55e-7 / 1.35e-7 / 1.35e-7, all of 3300 5.03e-8 / 4.93e-8 / 5.07e-8. Time
-// (us, calls in a loop), plain / so: 58.6 / 64.5, 253 / 277, and a step of 4001 particles
-// 12.7 / 12.4; folds of 16 4% less and errors up to 1% above the tiles'. The LJC laws'
+// sources (none up to 20), carry what a fold's sum leaves out into the next fold (Kahan's
+// summation) and, where direct_fine says so, compensate every exchange: a close pair's large
+// pull is rounded again with each later add. Rms errors against 64 bits, plain / so / tile:
+// 1500 targets of 65536 3.80e-8 / 3.66e-8 / 3.65e-8, 4000 of 131072 3.66e-8 / 3.46e-8 /
+// 3.49e-8, the same with a close companion for every particle 1.55e-7 / 1.35e-7 / 1.35e-7,
+// all of 3600 5.06e-8 / 4.93e-8 / 5.02e-8. Time (us, calls in a loop), plain / so: 55.5 /
+// 60.1, 236 / 257, a step of 4001 particles 11.6 / 12.2 (folds of 16 56.8, with errors to 2%
+// above the tiles'; of 8 61.1; with the low parts kept beside the sums 64.3). The LJC laws'
 // errors are those of their pair terms (1.2e-6 either way), and the VJPs and the jerk run
 // here up to 2432 particles, without folds.
 //
@@ -43,19 +44,10 @@ namespace nbody {
 constexpr int kDirectThreads = 256;
 constexpr int kDirectWarps = kDirectThreads / 32;
 constexpr int kDirectFold = 32;  // sources per register sum
-// Laws with finer sums (kFine): sources per register sum, the most that are added without
-// folds, and particles up to which the first two exchanges between lanes are plain
-constexpr int kFineFold = 12, kFineChain = 20, kFineFew = 2048;
+// Laws with finer sums (kFine): sources per register sum, and the most without folds
+constexpr int kFineFold = 12, kFineChain = 20;
 template <class L>
 constexpr int direct_chain() { return L::kFine ? kFineChain : kDirectFold; }
-
-// Adds a into the sum h with low part l: three operations of TwoSum's six, exact where h is
-// the larger one; where a is (a close pair's pull arrives), rounded once more.
-__device__ __forceinline__ void fold_add(float &h, float &l, float a) {
-  const float s = __fadd_rn(h, a);
-  l = __fadd_rn(l, __fsub_rn(a, __fsub_rn(s, h)));
-  h = s;
-}
 
 struct DirectArgs {
   const float4 *pos;  // sources (x, y, z, m)
@@ -81,6 +73,7 @@ struct DirectArgs {
   float4 *trace;     // drifted positions as well, or null
   float4 *x_lo;      // two-float state or null
   float4 *v_lo;
+  int fine;          // kFine: compensate every exchange between lanes (direct_fine)
   int pdl;           // host side
 };
 
@@ -153,20 +146,19 @@ __global__ void __launch_bounds__(kDirectThreads,
 #pragma unroll
         for (int c = 0; c < NS; ++c) {
           const int at = (r * NS + c) * kDirectThreads + tid;
-          if constexpr (L::kFine) {
-            float4 *f = reinterpret_cast<float4 *>(folded) + at;  // sums, then low parts
-            float4 t = make_float4(A[r][c].x, A[r][c].y, 0.0f, 0.0f);
-            if (!first) {
-              t = *f;
-              fold_add(t.x, t.z, A[r][c].x);
-              fold_add(t.y, t.w, A[r][c].y);
-            }
-            *f = t;
+          float2 *f = folded + at;
+          if (first) {
+            *f = A[r][c];
+            A[r][c] = make_float2(0.0f, 0.0f);
+          } else if (L::kFine) {
+            const float2 h = *f, s = __fadd2_rn(h, A[r][c]);
+            // what the sum leaves out, A - (s - h), goes into the next fold
+            A[r][c] = __ffma2_rn(__ffma2_rn(h, bcast(-1.0f), s), bcast(-1.0f), A[r][c]);
+            *f = s;
           } else {
-            float2 *f = folded + at;
-            *f = first ? A[r][c] : __fadd2_rn(*f, A[r][c]);
+            *f = __fadd2_rn(*f, A[r][c]);
+            A[r][c] = make_float2(0.0f, 0.0f);
           }
-          A[r][c] = make_float2(0.0f, 0.0f);
         }
     }
 #pragma unroll
@@ -193,14 +185,7 @@ __global__ void __launch_bounds__(kDirectThreads,
 #pragma unroll
       for (int c = 0; c < NS; ++c) {
         const int at = (r * NS + c) * kDirectThreads + tid;
-        if constexpr (L::kFine) {
-          float4 t = reinterpret_cast<const float4 *>(folded)[at];
-          fold_add(t.x, t.z, A[r][c].x);
-          fold_add(t.y, t.w, A[r][c].y);
-          A[r][c] = make_float2(t.x + t.z, t.y + t.w);
-        } else {
-          A[r][c] = __fadd2_rn(folded[at], A[r][c]);
-        }
+        A[r][c] = __fadd2_rn(folded[at], A[r][c]);
       }
   }
   // sums over the lanes: at each exchange a lane keeps half of its values (all of
@@ -219,7 +204,7 @@ __global__ void __launch_bounds__(kDirectThreads,
     }
 #pragma unroll
   for (int k = 0; k < (L::kFine ? V : V >> kComp); ++k) l[k] = 0.0f;
-  const bool fine = L::kFine && a.n > kFineFew;
+  const bool fine = L::kFine && a.fine;
   int base = 0, spare = 0;
 #pragma unroll
   for (int q = 0; q < 5; ++q) {

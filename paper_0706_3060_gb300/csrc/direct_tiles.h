@@ -31,8 +31,8 @@ struct DirectPlan {
 // a CTA has its SM to itself. Fitted to 1300 timings of 20 to 12000 targets and 2048 to
 // 131072 sources within 7% rms; the picks take 1% more than the best in the mean, e.g.
 // 1500 targets of 65536 in 16s and 3 slices 51 us (8s and 3 slices 69, 16s and 4 slices
-// 57). False where a thread's sum would have more than 32 folds at the most slices (n
-// above two million).
+// 57); fitted without gravity's folds of 12 sources, which add a tenth to `block`. False
+// where a thread would take more than 1024 sources at the most slices (n above two million).
 struct DirectCost {
   double block, fixed, alone, launch;  // us
   bool one;                            // one CTA on an SM
@@ -80,6 +80,15 @@ inline bool direct_plan(int law, bool pot, int64_t n_t, int64_t n, int sms, Dire
 // (us per step: gravity direct 13.1 at 4864, streamed 18.4 at 4865 where two direct waves
 // take 21; LJC direct 8.1 at 2432, 19.6 at 3000 where streamed takes 13.8).
 inline bool direct_all(int law, int64_t n, int sms) { return n <= (law == 0 ? 32 : 16) * sms; }
+
+// Whether gravity's sums compensate every exchange between lanes (0.6 us of a launch): where
+// with two plain ones the rms error of accelerations or potentials passes the tiles'. All n:
+// 0.99 and 1.00 of it at 2432, 0.99 and 1.01 at 2700, 1.02 and 1.01 at 3300 and 4095
+// (compensated 0.97 to 1.00), half of it from 4096 on; subsets of n sources, accelerations:
+// 0.97 at 8192, 1.00 at 12000, 1.01 at 16000 (0.96, 0.98, 1.00).
+inline bool direct_fine(bool subset, int64_t n) {
+  return subset ? n > 12000 : n > 2432 && n < 4096;
+}
 
 // The jerk and VJP laws (tile tables of tri_vjp.cu): 8 targets per CTA, 4 for the LJC
 // VJPs; mode 0 only.
