@@ -51,7 +51,9 @@ int grow(std::map<std::pair<int, cudaStream_t>, Arena> &tab, cudaStream_t s, siz
   std::lock_guard<std::mutex> lk(g_mu);
   Arena &a = tab[{dev, s}];
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (a.cap < bytes || !a.captured) NB_CUDA(cudaStreamIsCapturing(s, &cs));
+  // the legacy default stream is never captured, and asking costs its small calls 0.7 us
+  const bool legacy = s == nullptr || s == cudaStreamLegacy;
+  if (!legacy && (a.cap < bytes || !a.captured)) NB_CUDA(cudaStreamIsCapturing(s, &cs));
   if (cs != cudaStreamCaptureStatusNone && a.cap >= bytes) a.captured = true;
   if (a.cap < bytes) {
     if (cs != cudaStreamCaptureStatusNone)
