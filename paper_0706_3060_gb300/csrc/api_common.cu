@@ -438,8 +438,8 @@ bool plan_tri(int law, int64_t n, int sms, bool atomic_ok, Plan1 *out) {
   // partials are added exactly in fixed point with integer atomics (64 bytes a
   // particle), where the slots grow as n^2 (134 MB at 65536, 0.4 GB at 114688) and the
   // finalize with them: steps, us, here / there, 1145 / 1166 at 65536, 2554 / 2577 at
-  // 98304, 4524 / 4496 at 131072; forces with potential 1305 / 1462, 2911 / 3236, 5156 /
-  // 5575. Without softening, and with plain sums, those tiles keep slots too: from 163840
+  // 98304, 4524 / 4496 at 131072; forces with potential 1324 / 1462 (and
+  // before the finer sums, which take 1% more, 2911 / 3236, 5156 / 5575). Without softening, and with plain sums, those tiles keep slots too: from 163840
   // (forces, us, 1152 / 1201 at 65536, 4543 / 4550 at 131072, 18041 / 17820 at 262144).
   if (law == NBODY_LAW_GRAV && n >= (atomic_ok ? 114688 : 163840)) return false;
   if (bytes > sym_part_cap()) return false;

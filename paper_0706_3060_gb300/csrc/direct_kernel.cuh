@@ -25,12 +25,12 @@
 //
 // What bounds it: launch and latency up to about 1500 particles (one launch where the
 // tile path takes an interleave, a force and a finalize launch), then the packed FP32
-// unit (12 operations per gravity pair, one-sided; 72% of its issue slots at 6000 targets
-// of 65536). The pair symmetry is not used: it pays only where its partial sums cost less
-// than the pairs it saves (tri_kernel.cuh). Measured, against the tile kernels (us):
-// gravity steps at 1024 3.6 / 7.1, 2048 5.4 / 8.9, 4001 11.7 / 21.9; LJC 1024 4.4 / 8.2,
-// 2048 7.2 / 11.1; gravity subsets of 65536: 300 targets 20 / 40, 1500 52 / 183, 6000
-// 169 / 333; LJC 1500 103 / 230.
+// unit (12 operations per gravity pair, one-sided; 66% of its cycles at 1500 targets of
+// 65536, the folds among them). The pair symmetry is not used: it pays only where its
+// partial sums cost less than the pairs it saves (tri_kernel.cuh). Measured, against the
+// tile kernels (us): gravity steps at 1024 3.6 / 7.1, 2048 5.4 / 8.9, 4001 12.0 / 21.9; LJC
+// 1024 4.4 / 8.2, 2048 7.2 / 11.1; gravity subsets of 65536: 300 targets 16 / 40, 1500
+// 53 / 183, 6000 180 / 333; LJC 1500 99 / 230.
 #pragma once
 
 #include <cooperative_groups.h>

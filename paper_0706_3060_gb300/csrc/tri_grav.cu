@@ -13,8 +13,8 @@ using Fine = TriGrav<POT, PRECISE, true>;
 
 const TriDesc *tri_grav(int64_t n) {
   // Rows of 384 targets leave a small system more units for equal shares; rows of 512
-  // spend fewer instructions per pair on moving the sources. Kernel times (us), 384 /
-  // 512: 13.3 / 13.6 at 5000, 24.0 / 24.6 at 8192, 46.1 / 45.5 at 12288, 77.5 / 76.6 at
+  // spend fewer instructions per pair on moving the sources. Kernel times (us) with plain
+  // sums, 384 / 512: 13.3 / 13.6 at 5000, 24.0 / 24.6 at 8192, 46.1 / 45.5 at 12288, 77.5 / 76.6 at
   // 16384, 294 / 287 at 32768, 2170 / 2116 at 90000 (rows of 256: 15.7, 24.1, 48.5, 82.4,
   // 314, 2328).
   // The finer sums (tri_kernel.cuh, Sums) from 8192 on: below, the tiles' errors were twice

@@ -9,7 +9,7 @@
 // of 128 move the sources twice as often (LJC VJP: 1153 us at 32768 against 1065).
 // Per step with the finalize, against the block-pair tiles (us):
 //   Hermite 8192 45.8 / 79.2, 16384 161 / 215, 32768 616 / 685
-//   gravity reverse step 4096 20.0 / 27.4, 8192 47.3 / 61.7, 16384 166 / 185
+//   gravity reverse step 4096 20.4 / 27.4, 8192 47.3 / 61.7, 16384 166 / 185
 //   LJC reverse step 4096 32.5 / 46.3, 8192 77.6 / 105, 32768 1077 / 2186
 // The next group's sources are on their way in all but jerk (600 us at 32768 without,
 // 609 with).
